@@ -16,7 +16,8 @@
 // the transform, stages exchange through shared memory.
 //
 // Three arithmetic policies share the code:
-//   F64  complex128 (double2), native FP64 arithmetic;
+//   F64  complex128 (double2): FP64 storage, update, T(k) and sums; the line
+//        transforms in 64-bit fixed point (see the fixed-point section);
 //   F32  complex64 (float2), FP32 arithmetic;
 //   DF   complex stored as double-float pairs (hi + lo FP32, 16 bytes like
 //        complex128), arithmetic on the FP32 pipe with error-free
@@ -378,6 +379,83 @@ struct DF {
   };
 };
 
+// ============================================================ fixed point
+// The complex128 line transforms run on 64-bit integers.  GB300 issues two FP64
+// operations a clock and SM, but 128 integer additions and 64 multiply-adds of
+// 32 x 32 + 64 bits: an FP64 butterfly costs about ten times the clocks of the
+// same butterfly in fixed point, and a line of doubles needs no more than 64
+// bits once it is scaled by its largest element.
+//
+// A line (one column of a tile, or one z line) is scaled by the exponent E of
+// its largest component: v = x 2^(1081 - E), so |v| < 2^59 (2^58 for N = 96,
+// 192).  A radix-8 butterfly adds at most 3.5 bits (components stay below
+// 2^62.5), and the twiddles, held in Q61, give the product over 8, so every stage
+// starts below 2^59.5 again; the result is v 8^(S-1) 2^(E - 1081) with S stages.
+// Bits are dropped only where the transform has grown: the quantum of the last
+// stage is 2^-53 of the largest input for N = 512, against outputs that may be
+// 512 times larger.  Measured against a 64-bit transform, ten steps of 512^3
+// noise are off by 8.4e-16 (relative L2) in this form and by 8.6e-16 with the
+// FP64 butterflies.  Measured at 512^3 (FP64 butterflies, then this form): pass
+// A 12.03 and 4.54 ms, a y pass 5.31 and 1.48, the z pass 11.5 and 3.2.  Lines that do not fit (non-finite values, exponents near the ends of the
+// FP64 range) take the FP64 transform instead (fft_line).
+struct __align__(16) ic {
+  long long x, y;
+};
+// Twiddle exp(-2 pi i e / N) in Q61; each part as balanced limbs h 2^32 + l, l in [-2^31, 2^31).
+struct __align__(16) itw {
+  int rl, rh, il, ih;
+};
+constexpr int FX_R2_H = 1257966796, FX_R2_L = 102865788;  // 1 - sqrt(1/2)
+constexpr int FX_R3_H = 575416509, FX_R3_L = 1033546850;  // 1 - sqrt(3)/2
+struct sp {  // v = h 2^32 + l with signed l
+  int h, l;
+};
+__device__ __forceinline__ sp limbs(long long v) {
+  const int l = (int)v;
+  return sp{(int)(v >> 32) - (l >> 31), l};
+}
+__device__ __forceinline__ long long mw(int a, int b, long long c) { return (long long)a * (long long)b + c; }
+// round(v c / 2^64), c = ch 2^32 + cl
+__device__ __forceinline__ long long mulhi_c(long long v, int ch, int cl) {
+  const sp s = limbs(v);
+  return mw(s.h, ch, mw(s.l, ch, mw(s.h, cl, 1ll << 31)) >> 32);
+}
+// v sqrt(1/2) = v - v (1 - sqrt(1/2)) and v sqrt(3)/2 likewise: the factors as balanced limbs of c 2^64
+__device__ __forceinline__ long long mul_r2(long long v) { return v - mulhi_c(v, FX_R2_H, FX_R2_L); }
+__device__ __forceinline__ long long mul_r3(long long v) { return v - mulhi_c(v, FX_R3_H, FX_R3_L); }
+template <int DIR> __device__ __forceinline__ ic mul_w8(ic a) {
+  return DIR > 0 ? ic{mul_r2(a.x - a.y), mul_r2(a.x + a.y)} : ic{mul_r2(a.x + a.y), mul_r2(a.y - a.x)};
+}
+// a w / 8 (DIR < 0) or a conj(w) / 8, rounded
+template <int DIR> __device__ __forceinline__ ic mul_itw(ic a, itw w) {
+  const sp x = limbs(a.x), y = limbs(a.y);
+  const int il = DIR < 0 ? w.il : -w.il, ih = DIR < 0 ? w.ih : -w.ih;
+  const long long h = 1ll << 31;
+  const long long mr = mw(y.l, -ih, mw(y.h, -il, mw(x.l, w.rh, mw(x.h, w.rl, h))));
+  const long long mi = mw(y.l, w.rh, mw(y.h, w.rl, mw(x.l, ih, mw(x.h, il, h))));
+  return ic{mw(y.h, -ih, mw(x.h, w.rh, mr >> 32)), mw(y.h, w.rh, mw(x.h, ih, mi >> 32))};
+}
+// A double as v 2^(1081 - E) (bits below the quantum cut), its exponent field at most E.
+template <int K> __device__ __forceinline__ long long fx_in(double d, int E) {
+  const int hi = __double2hiint(d);
+  const unsigned long long m =
+      (((unsigned long long)((hi & 0xfffff) | 0x100000) << 32) | (unsigned)__double2loint(d)) << K;
+  const long long a = (long long)(m >> min(E - ((hi >> 20) & 0x7ff), 63));
+  const long long s = (long long)(hi >> 31);
+  return (a ^ s) - s;
+}
+// v 2^k as a double (k shifts the exponent field; the caller keeps it in range)
+__device__ __forceinline__ double fx_out(long long v, int k) {
+  const double f = __ll2double_rn(v);
+  const int h = __double2hiint(f);
+  return __hiloint2double(h ? h + (k << 20) : 0, __double2loint(f));
+}
+struct X64 {  // the transform policy of the fixed-point lines
+  using C = ic;
+  static constexpr int id = 3;
+};
+constexpr int FX_E_MIN = 64, FX_E_MAX = 1960;  // exponent fields of a line that runs in fixed point
+
 // ============================================================ FFT planning
 __host__ __device__ constexpr int ilog2c(int n) { return n <= 1 ? 0 : 1 + ilog2c(n / 2); }
 
@@ -457,6 +535,50 @@ template <int DIR, typename C> __device__ __forceinline__ void dft12(C* x) {
 #pragma unroll
   for (int k1 = 0; k1 < 3; ++k1) {
     C a = y[0][k1], b = y[1][k1], c = y[2][k1], d = y[3][k1];
+    dft4<DIR>(a, b, c, d);
+    x[k1] = a;
+    x[k1 + 3] = b;
+    x[k1 + 6] = c;
+    x[k1 + 9] = d;
+  }
+}
+// DFT-12 in fixed point: the halves are shifts, sqrt(3)/2 is mul_r3.
+template <int DIR> __device__ __forceinline__ void dft3(ic& a, ic& b, ic& c) {
+  const ic s = cadd(b, c), d = csub(b, c);
+  const ic m{a.x - (s.x >> 1), a.y - (s.y >> 1)};
+  const ic r = mul_i<DIR>(ic{mul_r3(d.x), mul_r3(d.y)});
+  a = cadd(a, s);
+  b = cadd(m, r);
+  c = csub(m, r);
+}
+template <int DIR> __device__ __forceinline__ void dft12(ic* x) {
+  ic y[4][3];
+#pragma unroll
+  for (int n2 = 0; n2 < 4; ++n2) {
+    ic a = x[n2], b = x[n2 + 4], c = x[n2 + 8];
+    dft3<DIR>(a, b, c);
+    y[n2][0] = a;
+    y[n2][1] = b;
+    y[n2][2] = c;
+  }
+  // a (sqrt(3)/2 + DIR i / 2) and a (1/2 + DIR i sqrt(3)/2)
+  auto w1 = [](ic a) {
+    return DIR > 0 ? ic{mul_r3(a.x) - (a.y >> 1), mul_r3(a.y) + (a.x >> 1)}
+                   : ic{mul_r3(a.x) + (a.y >> 1), mul_r3(a.y) - (a.x >> 1)};
+  };
+  auto w2 = [](ic a) {
+    return DIR > 0 ? ic{(a.x >> 1) - mul_r3(a.y), (a.y >> 1) + mul_r3(a.x)}
+                   : ic{(a.x >> 1) + mul_r3(a.y), (a.y >> 1) - mul_r3(a.x)};
+  };
+  y[1][1] = w1(y[1][1]);
+  y[1][2] = w2(y[1][2]);
+  y[2][1] = w2(y[2][1]);
+  y[2][2] = mul_i<DIR>(w1(y[2][2]));  // w12^4 = i w12
+  y[3][1] = mul_i<DIR>(y[3][1]);
+  y[3][2] = ic{-y[3][2].x, -y[3][2].y};
+#pragma unroll
+  for (int k1 = 0; k1 < 3; ++k1) {
+    ic a = y[0][k1], b = y[1][k1], c = y[2][k1], d = y[3][k1];
     dft4<DIR>(a, b, c, d);
     x[k1] = a;
     x[k1 + 3] = b;
@@ -606,6 +728,14 @@ __device__ __forceinline__ void scaled_bfly8(double2 (&x)[8], const double2* __r
   x[7] = axpy2(E3, -kap, O3);
 }
 
+// The twiddle table entry of a policy.
+template <class A> struct TwOf {
+  using type = typename A::C;
+};
+template <> struct TwOf<X64> {
+  using type = itw;
+};
+
 // One Stockham stage on the register-resident canonical set v[m] = x[t + m N/E].
 // Butterfly b = t + u N/E (u < E/RAD) takes x[b + r N/RAD] = v[u + r (E/RAD)],
 // multiplies input r by w_N^{(b mod NS) r N/(NS RAD)}, and applies DFT_RAD.
@@ -615,7 +745,7 @@ __device__ __forceinline__ void scaled_bfly8(double2 (&x)[8], const double2* __r
 // inverse y pass).
 template <class A, int N, int R, int RAD, int NS, int DIR, bool LAST, bool TWC = false>
 __device__ __forceinline__ void stage_compute(typename A::C (&v)[FftPlan<N, R>::E], int t,
-                                              const typename A::C* __restrict__ tw) {
+                                              const typename TwOf<A>::type* __restrict__ tw) {
   using C = typename A::C;
   constexpr int E = FftPlan<N, R>::E;
   constexpr int NB = E / RAD;
@@ -636,7 +766,15 @@ __device__ __forceinline__ void stage_compute(typename A::C (&v)[FftPlan<N, R>::
     if (NS > 1) {
       const int b = t + u * (N / E);
       const int e0 = (b % NS) * (N / (NS * RAD));
-      if constexpr (TWC && A::id == 1) {
+      if constexpr (A::id == 3) {
+        // the product over 8 (see the fixed-point section), r = 0 included
+#pragma unroll
+        for (int r = 1; r < RAD; ++r) {
+          const int4 q = __ldg(reinterpret_cast<const int4*>(tw + e0 * r));
+          x[r] = mul_itw<DIR>(x[r], itw{q.x, q.y, q.z, q.w});
+        }
+        x[0] = ic{(x[0].x + 4) >> 3, (x[0].y + 4) >> 3};
+      } else if constexpr (TWC && A::id == 1) {
         // w = exp(-2 pi i e0 / N) from sincospif, its powers by products
         // (a few ulp of FP32, like the rounding of the transform itself)
         float sn, cs;
@@ -686,7 +824,7 @@ __device__ __forceinline__ void stage_exchange(C (&v)[FftPlan<N, R>::E], int t, 
 
 template <class A, int N, int R, int DIR, int I, bool TWC, class Acc>
 __device__ __forceinline__ void fft_stages(typename A::C (&v)[FftPlan<N, R>::E], int t,
-                                           const typename A::C* __restrict__ tw, Acc& acc) {
+                                           const typename TwOf<A>::type* __restrict__ tw, Acc& acc) {
   using PL = FftPlan<N, R>;
   if constexpr (I < PL::S) {
     constexpr int RAD = PL::radix(I);
@@ -697,12 +835,57 @@ __device__ __forceinline__ void fft_stages(typename A::C (&v)[FftPlan<N, R>::E],
   }
 }
 
+// The FP64 transform of the complex128 lines that fixed point does not cover,
+// out of line so that its registers and code stay out of the common path.
+template <int N, int DIR, class Acc>
+__device__ __noinline__ void fft_line_f64(double2* v, int t, const double2* __restrict__ tw, Acc acc) {
+  double2 w[FftPlan<N>::E];
+#pragma unroll
+  for (int m = 0; m < FftPlan<N>::E; ++m) w[m] = v[m];
+  fft_stages<F64, N, 0, DIR, 0, false>(w, t, tw, acc);
+#pragma unroll
+  for (int m = 0; m < FftPlan<N>::E; ++m) v[m] = w[m];
+}
+
+// A complex128 line in fixed point: scaled by the line's largest component,
+// transformed on integers, returned as doubles.
+template <int N, int DIR, class Acc>
+__device__ __forceinline__ void fft_line_fx(double2 (&v)[FftPlan<N>::E], int t, const double2* __restrict__ tw,
+                                            Acc& acc) {
+  using PL = FftPlan<N>;
+  constexpr int K = PL::R3 ? 5 : 6;
+  int mx = 0;
+#pragma unroll
+  for (int m = 0; m < PL::E; ++m)
+    mx = max(mx, max(__double2hiint(v[m].x) & 0x7fffffff, __double2hiint(v[m].y) & 0x7fffffff));
+  const bool odd = mx >= (FX_E_MAX << 20) || (mx != 0 && mx < (FX_E_MIN << 20));
+  if (acc.line_max(mx, odd, t)) {
+    double2 w[PL::E];
+#pragma unroll
+    for (int m = 0; m < PL::E; ++m) w[m] = v[m];
+    fft_line_f64<N, DIR>(w, t, tw, acc);
+#pragma unroll
+    for (int m = 0; m < PL::E; ++m) v[m] = w[m];
+    return;
+  }
+  const int E = max(mx >> 20, FX_E_MIN);  // an all-zero line: any scale
+  ic x[PL::E];
+#pragma unroll
+  for (int m = 0; m < PL::E; ++m) x[m] = ic{fx_in<K>(v[m].x, E), fx_in<K>(v[m].y, E)};
+  auto xacc = acc.template as<ic>();
+  fft_stages<X64, N, 0, DIR, 0, false>(x, t, reinterpret_cast<const itw*>(tw + 3 * N), xacc);
+  const int k = E - 1075 - K + 3 * (PL::S - 1);
+#pragma unroll
+  for (int m = 0; m < PL::E; ++m) v[m] = double2{fx_out(x[m].x, k), fx_out(x[m].y, k)};
+}
+
 // Unnormalised length-N DFT, sign DIR, canonical layout in and out, radix
-// schedule R.
+// schedule R.  Complex128 lines run in fixed point.
 template <class A, int N, int DIR, class Acc, bool TWC = false, int R = 0>
 __device__ __forceinline__ void fft_line(typename A::C (&v)[FftPlan<N, R>::E], int t,
                                          const typename A::C* __restrict__ tw, Acc& acc) {
-  fft_stages<A, N, R, DIR, 0, TWC>(v, t, tw, acc);
+  if constexpr (A::id == 0) fft_line_fx<N, DIR>(v, t, tw, acc);
+  else fft_stages<A, N, R, DIR, 0, TWC>(v, t, tw, acc);
 }
 
 // Shared-memory views. Tile of CW columns of a strided axis: [pos][col] with a
@@ -712,11 +895,34 @@ __device__ __forceinline__ void fft_line(typename A::C (&v)[FftPlan<N, R>::E], i
 // but was measured slower at 512^3, by the index arithmetic it adds to every
 // access, so the tiles are unpadded.)  The columns of a tile interleave across
 // all warps of the CTA, so an exchange synchronises the whole CTA.
-template <typename C, int CW, int PITCH> struct AccTile {
+// line_max (complex128): reduces mx over the threads of a line and returns
+// whether any line that shares the tile's barriers is `odd`.  The partial
+// maxima go to one of two buffers in turn, so that one barrier suffices.
+template <typename C, int CW, int T> struct AccTile {
+  static constexpr int G = CW >= 32 ? 1 : (32 / CW < T ? 32 / CW : T);  // threads of a column in a warp
+  static constexpr int ROWS = T / G;                                       // partial maxima of a column
+  static constexpr int MAXN = 2 * ROWS * CW;
   C* sm;
   int col;
-  __device__ __forceinline__ C& at(int pos) { return sm[pos * PITCH + col]; }
+  int* mxs;
+  int flip;
+  __device__ __forceinline__ AccTile(C* s, int c, int* m = nullptr, int f = 0) : sm(s), col(c), mxs(m), flip(f) {}
+  template <typename D> __device__ __forceinline__ AccTile<D, CW, T> as() const {
+    return AccTile<D, CW, T>(reinterpret_cast<D*>(sm), col);
+  }
+  __device__ __forceinline__ C& at(int pos) { return sm[pos * CW + col]; }
   __device__ __forceinline__ void sync() { __syncthreads(); }
+  __device__ __forceinline__ bool line_max(int& mx, bool odd, int t) {
+#pragma unroll
+    for (int o = CW; o < CW * G; o <<= 1) mx = max(mx, __shfl_xor_sync(0xffffffffu, mx, o));
+    int* b = mxs + flip;
+    flip = flip ? 0 : ROWS * CW;
+    if (t % G == 0) b[t / G * CW + col] = mx;
+    const bool any = __syncthreads_or(odd);
+#pragma unroll 8
+    for (int r = 0; r < ROWS; ++r) mx = max(mx, b[r * CW + col]);
+    return any;
+  }
 };
 // One contiguous line of T threads, padded by one element every 2^PS elements
 // (128 bytes for the radix-8 schedule; every E elements for the two-stage one,
@@ -724,14 +930,40 @@ template <typename C, int CW, int PITCH> struct AccTile {
 // synchronise independently: a warp barrier when lines do not straddle warps
 // (T <= 32), else the named barrier 1 + line (T threads).
 template <typename C, int PS, int T> struct AccLine {
+  static constexpr int WARPS = T > 32 ? T / 32 : 1;
+  static constexpr int MAXN = 2 * WARPS;  // per line
   C* sm;
   int line;
+  int* mxs;
+  int flip;
+  __device__ __forceinline__ AccLine(C* s, int l, int* m = nullptr, int f = 0) : sm(s), line(l), mxs(m), flip(f) {}
+  template <typename D> __device__ __forceinline__ AccLine<D, PS, T> as() const {
+    return AccLine<D, PS, T>(reinterpret_cast<D*>(sm), line);
+  }
   __device__ __forceinline__ C& at(int pos) { return sm[pos + (pos >> PS)]; }
   __device__ __forceinline__ void sync() {
     if constexpr (T <= 32) {
       __syncwarp();
     } else {
       asm volatile("bar.sync %0, %1;" ::"r"(1 + line), "r"(T) : "memory");
+    }
+  }
+  // the lines of a warp (T <= 32) take the same path, else each line its own
+  __device__ __forceinline__ bool line_max(int& mx, bool odd, int t) {
+    if constexpr (T <= 32) {
+#pragma unroll
+      for (int o = 1; o < T; o <<= 1) mx = max(mx, __shfl_xor_sync(0xffffffffu, mx, o));
+      return __any_sync(0xffffffffu, odd);
+    } else {
+      if (odd) mx = 0x7fffffff;
+      mx = __reduce_max_sync(0xffffffffu, mx);
+      int* b = mxs + line * MAXN + flip;
+      flip = flip ? 0 : WARPS;
+      if (t % 32 == 0) b[t / 32] = mx;
+      sync();
+#pragma unroll
+      for (int r = 0; r < WARPS; ++r) mx = max(mx, b[r]);
+      return mx == 0x7fffffff;
     }
   }
 };
@@ -1004,7 +1236,9 @@ __device__ __forceinline__ void fft_strided_body(typename A::C* W, const typenam
   C v[PL::E];
 #pragma unroll
   for (int m = 0; m < PL::E; ++m) v[m] = W[base + (int64_t)(t + m * PL::T) * stride];
-  AccTile<C, YC, YC> acc{sm, col};
+  using AT = AccTile<C, YC, PL::T>;
+  __shared__ int mxs[A::id == 0 ? AT::MAXN : 1];
+  AT acc{sm, col, mxs};
   // complex64 inverse y pass and the two-stage schedule: computed twiddles
   // (measured faster there; the forward y pass of schedule 0 is faster with
   // the table)
@@ -1053,7 +1287,9 @@ __device__ __forceinline__ void zpass_body(typename A::C* W, const typename A::C
   static_assert(PL::T <= 32 || LINES <= 15, "one named barrier per line");
   constexpr int PS = R == 0 ? SH::PAD_SHIFT : SH::PAD_SHIFT_R1;
   constexpr int LP = R == 0 ? SH::LPAD : SH::LPAD_R1;
-  AccLine<C, PS, PL::T> acc{sm + l * LP, l};
+  using AL = AccLine<C, PS, PL::T>;
+  __shared__ int mxs[A::id == 0 ? AL::MAXN * LINES : 1];
+  AL acc{sm + l * LP, l, mxs};
   typename A::Pars pacc;
 #pragma unroll
   for (int g = 0; g < ZG; ++g) {
@@ -1105,14 +1341,17 @@ __global__ void __launch_bounds__(FftPlan<N, R>::T * ZLines<A, N, R>::value) k_z
 template <class A, int N, int STATS, int XC>
 __device__ __forceinline__ void update_x_core(typename A::C (&v)[FftPlan<N>::E], const typename A::C (&ps)[FftPlan<N>::E],
                                               const typename A::U (&cf)[FftPlan<N>::E], int t, int col, int64_t base,
-                                              typename A::C* W, typename A::C* __restrict__ psi, const UpdParams& upar,
+                                              typename A::C* W, typename A::C* __restrict__ psi,
+                                              const typename A::U* __restrict__ uin, const UpdParams& upar,
                                               const typename A::VT* __restrict__ V, const double* __restrict__ scale,
                                               const float* __restrict__ scale_f, const typename A::C* __restrict__ tw,
                                               typename A::C* sm, typename A::Acc& nacc, typename A::Full& facc) {
   using C = typename A::C;
   using SH = Shape<A, N>;
   constexpr int64_t S = (int64_t)N * N;
-  AccTile<C, XC, XC> acc{sm, col};
+  using AT = AccTile<C, XC, SH::T>;
+  __shared__ int mxs[A::id == 0 ? AT::MAXN : 1];
+  AT acc{sm, col, mxs};
   fft_line<A, N, +1>(v, t, tw, acc);
   const bool scaled = scale != nullptr;
   typename A::S s{};
@@ -1120,7 +1359,9 @@ __device__ __forceinline__ void update_x_core(typename A::C (&v)[FftPlan<N>::E],
 #pragma unroll
   for (int m = 0; m < SH::E; ++m) {
     const int64_t idx = base + (t + m * SH::T) * S;
-    C nw = A::update(ps[m], v[m], A::coef_from(cf[m], upar));
+    C nw;
+    if constexpr (A::id == 0) nw = A::update(psi[idx], v[m], A::coef_from(uin[idx], upar));
+    else nw = A::update(ps[m], v[m], A::coef_from(cf[m], upar));
     if (scaled) nw = cscale(nw, s);
     psi[idx] = nw;
     v[m] = nw;
@@ -1152,13 +1393,15 @@ __device__ __forceinline__ void update_x_body(typename A::C* W, typename A::C* _
   U cf[SH::E];
 #pragma unroll
   for (int m = 0; m < SH::E; ++m) v[m] = W[base + (t + m * SH::T) * S];
+  if constexpr (A::id != 0) {  // (the fixed-point transforms leave no registers to hold them)
 #pragma unroll
-  for (int m = 0; m < SH::E; ++m) ps[m] = psi[base + (t + m * SH::T) * S];
+    for (int m = 0; m < SH::E; ++m) ps[m] = psi[base + (t + m * SH::T) * S];
 #pragma unroll
-  for (int m = 0; m < SH::E; ++m) cf[m] = uin[base + (t + m * SH::T) * S];
+    for (int m = 0; m < SH::E; ++m) cf[m] = uin[base + (t + m * SH::T) * S];
+  }
   typename A::Acc nacc;
   typename A::Full facc;
-  update_x_core<A, N, STATS, XC>(v, ps, cf, t, col, base, W, psi, upar, V, scale, scale_f, tw, sm, nacc, facc);
+  update_x_core<A, N, STATS, XC>(v, ps, cf, t, col, base, W, psi, uin, upar, V, scale, scale_f, tw, sm, nacc, facc);
   if constexpr (STATS == STATS_NORM) norm_reduce_store<A>(nacc, part);
   if constexpr (STATS == STATS_FULL) full_store<A>(facc, part);
 }
@@ -1210,7 +1453,9 @@ k_forward_x(const typename A::C* src, typename A::C* W, typename A::C* psi_out, 
 #pragma unroll
     for (int m = 0; m < SH::E; ++m) psi_out[base + (t + m * SH::T) * S] = v[m];
   }
-  AccTile<C, SH::XCOLS, SH::XPITCH> acc{sm, col};
+  using AT = AccTile<C, SH::XCOLS, SH::T>;
+  __shared__ int mxs[A::id == 0 ? AT::MAXN : 1];
+  AT acc{sm, col, mxs};
   fft_line<A, N, -1>(v, t, tw, acc);
 #pragma unroll
   for (int m = 0; m < SH::E; ++m) W[base + (t + m * SH::T) * S] = v[m];
@@ -1319,7 +1564,9 @@ k_project_x(const typename A::C* __restrict__ src, LowerPtrs lower, const double
     if constexpr (STATS == STATS_NORM) nacc.add_norm(p);
     if constexpr (STATS == STATS_FULL) facc.add(p, V[idx]);
   }
-  AccTile<C, SH::XCOLS, SH::XPITCH> acc{sm, col};
+  using AT = AccTile<C, SH::XCOLS, SH::T>;
+  __shared__ int mxs[A::id == 0 ? AT::MAXN : 1];
+  AT acc{sm, col, mxs};
   fft_line<A, N, -1>(v, t, tw, acc);
 #pragma unroll
   for (int m = 0; m < SH::E; ++m) W[base + (t + m * SH::T) * S] = v[m];

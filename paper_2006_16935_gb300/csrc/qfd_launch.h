@@ -51,6 +51,31 @@ inline void scaled_twiddle_table(int64_t n, const double2* tw, double2* out) {
     }
 }
 
+// The twiddles of the fixed-point complex128 lines: exp(-2 pi i e / n) in Q61,
+// each part split into balanced limbs h 2^32 + l (l signed), as int4
+// {rl, rh, il, ih}; n entries of 16 bytes after the scaled block.  Angles are
+// reduced to the first octant in integers and evaluated in long double.
+inline void fixed_twiddle_table(int64_t n, double2* out) {
+  using LD = long double;
+  const LD pi = 3.14159265358979323846264338327950288L;
+  auto limbs = [](LD x, int32_t* l, int32_t* h) {
+    const int64_t v = (int64_t)std::llrint(std::ldexp(x, 61));
+    *l = (int32_t)(uint32_t)(uint64_t)v;
+    *h = (int32_t)((v - (int64_t)*l) / ((int64_t)1 << 32));
+  };
+  for (int64_t e = 0; e < n; ++e) {
+    const int64_t q = (4 * e) / n, rem = 4 * e - q * n;  // angle pi/2 (q + rem/n)
+    const bool low = 2 * rem <= n;
+    const LD phi = pi / 2 * (LD)(low ? rem : n - rem) / (LD)n;
+    const LD c = low ? std::cos(phi) : std::sin(phi), s = low ? std::sin(phi) : std::cos(phi);
+    const LD re[4] = {c, -s, -c, s}, im[4] = {-s, -c, s, c};
+    int32_t w[4];
+    limbs(re[q], &w[0], &w[1]);
+    limbs(im[q], &w[2], &w[3]);
+    std::memcpy(out + e, w, sizeof(w));
+  }
+}
+
 struct KinParams;
 struct UpdParams;
 struct BatchY;
