@@ -1002,6 +1002,14 @@ template <typename C, int PS, int T> struct AccLine {
 #ifndef QFD_LINE_TARGET8
 #define QFD_LINE_TARGET8 128
 #endif
+// Resident CTAs per SM asked of the compiler for the complex128 kernels: 1024
+// threads (64 registers each).  The fixed-point transforms are chains of integer
+// operations, bound by how many warps hide their latency: at 512^3 with 512 /
+// 768 / 1024 threads an SM the y pass takes 1.49 / 1.32 / 1.26 ms, the z pass
+// 3.20 / 2.82 / 2.58 and pass A 4.54 / 3.98 / 3.76 (at most 32 bytes spilled).
+__host__ __device__ constexpr int f64_ctas(int threads) {
+  return 1024 / threads < 1 ? 1 : (1024 / threads > 8 ? 8 : 1024 / threads);
+}
 template <int N, int CMIN> struct TileCols {
   static constexpr int T = N / FftPlan<N>::E;
   static constexpr int C0 = (QFD_TILE_TARGET / T > CMIN) ? QFD_TILE_TARGET / T : CMIN;
@@ -1251,7 +1259,7 @@ __device__ __forceinline__ void fft_strided_body(typename A::C* W, const typenam
 // many warps in flight), the 16-byte arithmetics take what their registers allow.
 template <class A, int N, int YC> struct YOcc {
   static constexpr int THREADS = N / FftPlan<N>::E * YC;
-  static constexpr int B0 = A::id == 1 ? 1536 / THREADS : 1;
+  static constexpr int B0 = A::id == 1 ? 1536 / THREADS : A::id == 0 ? f64_ctas(THREADS) : 1;
   static constexpr int value = B0 < 1 ? 1 : (B0 > 8 ? 8 : B0);
 };
 template <class A, int N, int DIR, int YC, int R = 0>
@@ -1322,7 +1330,9 @@ template <class A, int N, int R> struct ZLines {
   static constexpr int value = R == 0 ? Shape<A, N>::LINES : Shape<A, N>::LINES_R1;
 };
 template <class A, int N, bool PARSEVAL, int ZG, int R = 0>
-__global__ void __launch_bounds__(FftPlan<N, R>::T * ZLines<A, N, R>::value) k_zpass(const __grid_constant__ BatchZ b) {
+__global__ void __launch_bounds__(FftPlan<N, R>::T * ZLines<A, N, R>::value,
+                                  A::id == 0 && ZG == 1 ? f64_ctas(FftPlan<N, R>::T * ZLines<A, N, R>::value) : 1)
+k_zpass(const __grid_constant__ BatchZ b) {
   using C = typename A::C;
   const int i = blockIdx.y;
   zpass_body<A, N, PARSEVAL, ZG, R, ZLines<A, N, R>::value>(static_cast<C*>(b.W[i]), static_cast<const C*>(b.tw[i]),
@@ -1409,7 +1419,8 @@ __device__ __forceinline__ void update_x_body(typename A::C* W, typename A::C* _
 // of `scaled` is set.  The half-width tiles (XC < XCOLS) are compiled for two
 // resident CTAs per SM.
 template <class A, int N, int STATS, int XC>
-__global__ void __launch_bounds__(N / FftPlan<N>::E * XC, XC < Shape<A, N>::XCOLS ? 2 : 1)
+__global__ void __launch_bounds__(N / FftPlan<N>::E * XC,
+                                  A::id == 0 ? f64_ctas(N / FftPlan<N>::E * XC) : XC < Shape<A, N>::XCOLS ? 2 : 1)
 k_update_x(const __grid_constant__ BatchU b, uint32_t scaled) {
   using C = typename A::C;
   const int i = blockIdx.y;
@@ -1423,7 +1434,7 @@ k_update_x(const __grid_constant__ BatchU b, uint32_t scaled) {
 // psi_out) into W; partials per STATS of the scaled input.  src may alias W
 // (each CTA reads its whole tile before writing it).
 template <class A, int N, int STATS>
-__global__ void __launch_bounds__(Shape<A, N>::XTHREADS)
+__global__ void __launch_bounds__(Shape<A, N>::XTHREADS, A::id == 0 ? f64_ctas(Shape<A, N>::XTHREADS) : 1)
 k_forward_x(const typename A::C* src, typename A::C* W, typename A::C* psi_out, const typename A::VT* __restrict__ V,
             const double* __restrict__ scale, const float* __restrict__ scale_f, const typename A::C* __restrict__ tw,
             double* __restrict__ part) {
@@ -1518,7 +1529,7 @@ k_gs_dots(const typename A::C* __restrict__ psi, LowerPtrs lower, int k, int par
 // LOWER: whether there are lower states (k > 0); the parity-only instance
 // carries no Gram-Schmidt code at all.
 template <class A, int N, int STATS, bool LOWER = true>
-__global__ void __launch_bounds__(Shape<A, N>::XTHREADS)
+__global__ void __launch_bounds__(Shape<A, N>::XTHREADS, A::id == 0 && !LOWER ? f64_ctas(Shape<A, N>::XTHREADS) : 1)
 k_project_x(const typename A::C* __restrict__ src, LowerPtrs lower, const double* __restrict__ sums, int k, int parity,
             int offgrid, typename A::C* __restrict__ dst, typename A::C* __restrict__ W,
             const typename A::VT* __restrict__ V,
