@@ -46,8 +46,9 @@ namespace qfd {
 
 // Fixed-order sums of per-CTA partials, then the derived scalars of `op`.
 __global__ void __launch_bounds__(FIN_THREADS)
-k_finalize_op(const double* __restrict__ part, int nq, int count, double* __restrict__ scal, float* __restrict__ scalf,
+k_finalize_op(const double* part, int nq, int count, double* scal, float* scalf,
               int op) {
+  pdl_begin();
   __shared__ double red[32];
   __shared__ double sums[2 * MAX_LOWER];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -167,6 +168,7 @@ __device__ __forceinline__ uint64_t splitmix64(uint64_t x) {
 
 template <class A>
 __global__ void k_fill_uniform(typename A::C* __restrict__ psi, int64_t n3, uint64_t seed) {
+  pdl_begin();
   const uint64_t base = seed * 0x9E3779B97F4A7C15ull;
   for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n3; i += (int64_t)gridDim.x * blockDim.x) {
     const uint64_t z0 = splitmix64(base ^ (uint64_t)(2 * i)), z1 = splitmix64(base ^ (uint64_t)(2 * i + 1));
@@ -207,7 +209,8 @@ __device__ __forceinline__ int64_t lat_wrap(Lat L, int64_t c) {
 // axis k and F_other that of the two other axes.
 template <class A>
 __global__ void __launch_bounds__(256)
-k_observables(const typename A::C* __restrict__ psi, Lat L, int offgrid, double half, double* __restrict__ part) {
+k_observables(const typename A::C* psi, Lat L, int offgrid, double half, double* __restrict__ part) {
+  pdl_begin();
   const int64_t n = L.n, n3 = n * n * n;
   const double cen = offgrid ? 0.5 * (double)(n - 1) : (double)(n / 2);
   double acc[NOBS];
@@ -248,7 +251,8 @@ k_observables(const typename A::C* __restrict__ psi, Lat L, int offgrid, double 
 }
 
 template <class AI, class AO>
-__global__ void k_convert(const typename AI::C* __restrict__ in, typename AO::C* __restrict__ out, int64_t n3) {
+__global__ void k_convert(const typename AI::C* in, typename AO::C* out, int64_t n3) {
+  pdl_begin();
   for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n3; i += (int64_t)gridDim.x * blockDim.x)
     out[i] = AO::from_d2(AI::to_d2(in[i]));
 }
@@ -259,7 +263,7 @@ __global__ void k_convert(const typename AI::C* __restrict__ in, typename AO::C*
 // Eq. HK0_momentum_space_1): c (6 psi - the sum of the six neighbours) with
 // c = 1 / (2 M A^2).  `self` receives psi at idx.
 template <class A>
-__device__ __forceinline__ typename A::C fdtd_sum(const typename A::C* __restrict__ psi, int64_t idx, Lat L,
+__device__ __forceinline__ typename A::C fdtd_sum(const typename A::C* psi, int64_t idx, Lat L,
                                                   typename A::C& self) {
   using C = typename A::C;
   const int64_t n = L.n, n2 = n * n;
@@ -276,7 +280,7 @@ __device__ __forceinline__ typename A::C fdtd_sum(const typename A::C* __restric
   return s;
 }
 template <class A>
-__device__ __forceinline__ typename A::C fdtd_hk(const typename A::C* __restrict__ psi, int64_t idx, Lat L,
+__device__ __forceinline__ typename A::C fdtd_hk(const typename A::C* psi, int64_t idx, Lat L,
                                                  typename A::S c, typename A::C& self) {
   const typename A::C s = fdtd_sum<A>(psi, idx, L, self);
   return cscale(csub(cscale(self, A::scalar(6.0)), s), c);
@@ -289,9 +293,10 @@ __device__ __forceinline__ typename A::C fdtd_hk(const typename A::C* __restrict
 // lattices (the stencil reads neighbours).
 template <class A, int STATS>
 __global__ void __launch_bounds__(256)
-k_fdtd_update(const typename A::C* __restrict__ psi, typename A::C* __restrict__ out,
+k_fdtd_update(const typename A::C* psi, typename A::C* __restrict__ out,
               const typename A::K* __restrict__ coef, const typename A::VT* __restrict__ V,
-              const double* __restrict__ scale, const float* __restrict__ scale_f, Lat L, double* __restrict__ part) {
+              const double* scale, const float* scale_f, Lat L, double* __restrict__ part) {
+  pdl_begin();
   using C = typename A::C;
   const int64_t n3 = L.n * L.n * L.n;
   const bool scaled = scale != nullptr;
@@ -319,7 +324,8 @@ k_fdtd_update(const typename A::C* __restrict__ psi, typename A::C* __restrict__
 // Per-CTA partials of <psi|H_K(0)|psi> (FP64 accumulation).
 template <class A>
 __global__ void __launch_bounds__(256)
-k_fdtd_energy(const typename A::C* __restrict__ psi, Lat L, typename A::S c, double* __restrict__ part) {
+k_fdtd_energy(const typename A::C* psi, Lat L, typename A::S c, double* __restrict__ part) {
+  pdl_begin();
   using C = typename A::C;
   const int64_t n3 = L.n * L.n * L.n;
   double e = 0.0;
@@ -634,8 +640,7 @@ const void* psi_tmap(qfd_plan_t pl, const void* p) {
 
 qfd_status finalize(qfd_plan_t pl, const double* part, int nq, int count, int op) {
   QFD_RUN(PASS_FINALIZE,
-          (k_finalize_op<<<1, FIN_THREADS, 0, pl->st>>>(part, nq, count, pl->scal, pl->scalf, op),
-           cudaGetLastError()));
+          pdl_launch(k_finalize_op, 1, FIN_THREADS, 0, pl->st, part, nq, count, pl->scal, pl->scalf, op));
   return QFD_OK;
 }
 
@@ -746,9 +751,8 @@ qfd_status take_snapshot(qfd_plan_t pl) {
   }
   sp[1] = oldest;
   pl->snap_t[0] = pl->t[0];
-  QFD_RUN(PASS_OTHER, (k_scale_copy<A><<<grid_for(pl->n3), 256, 0, pl->st>>>(
-                           psi_of<A>(pl, 1), psi_of<A>(pl, 0), pl->n3, pl->pending ? pl->scal + SC_SCALE : nullptr),
-                       cudaGetLastError()));
+  QFD_RUN(PASS_OTHER, pdl_launch(k_scale_copy<A>, grid_for(pl->n3), 256, 0, pl->st,  psi_of<A>(pl, 1),
+                                 psi_of<A>(pl, 0), pl->n3, pl->pending ? pl->scal + SC_SCALE : nullptr));
   return QFD_OK;
 }
 
@@ -758,10 +762,9 @@ template <class A>
 qfd_status fdtd_update(qfd_plan_t pl, int s, int stats) {
   const double* scale = pl->pending ? pl->scal + SC_SCALE : nullptr;
   auto go = [&](auto kern) -> cudaError_t {
-    kern<<<GS_BLOCKS, 256, 0, pl->st>>>(psi_of<A>(pl, s), spare_of<A>(pl),
-                                        static_cast<const typename A::K*>(coef_of<A>(pl)), v_of<A>(pl), scale, pl->scalf,
-                                        Lat{pl->p.n, pl->lg}, pl->partA);
-    return cudaGetLastError();
+    return pdl_launch(kern, GS_BLOCKS, 256, 0, pl->st, psi_of<A>(pl, s), spare_of<A>(pl),
+                      static_cast<const typename A::K*>(coef_of<A>(pl)), v_of<A>(pl), scale, pl->scalf,
+                      Lat{pl->p.n, pl->lg}, pl->partA);
   };
   auto launch = [&]() -> cudaError_t {
     if (stats == STATS_FULL) return go(k_fdtd_update<A, STATS_FULL>);
@@ -780,8 +783,8 @@ qfd_status fdtd_update(qfd_plan_t pl, int s, int stats) {
 template <class A>
 qfd_status fdtd_energy_partials(qfd_plan_t pl, int s) {
   const typename A::S c = host_scalar<A>(pl->fdtd_c);
-  QFD_RUN(PASS_ZKIN, (k_fdtd_energy<A><<<GS_BLOCKS, 256, 0, pl->st>>>(psi_of<A>(pl, s), Lat{pl->p.n, pl->lg}, c, pl->partC),
-                      cudaGetLastError()));
+  QFD_RUN(PASS_ZKIN, pdl_launch(k_fdtd_energy<A>, GS_BLOCKS, 256, 0, pl->st, psi_of<A>(pl, s), Lat{pl->p.n,
+                                pl->lg}, c, pl->partC));
   pl->nC = GS_BLOCKS;
   return QFD_OK;
 }
@@ -830,8 +833,8 @@ qfd_status step_once(qfd_plan_t pl, int s, int check) {
 template <class A>
 qfd_status materialize(qfd_plan_t pl, int s) {
   if (pl->pending) {
-    QFD_RUN(PASS_OTHER, (k_scale<A><<<grid_for(pl->n3), 256, 0, pl->st>>>(psi_of<A>(pl, s), pl->n3, pl->scal + SC_SCALE, 0),
-                         cudaGetLastError()));
+    QFD_RUN(PASS_OTHER, pdl_launch(k_scale<A>, grid_for(pl->n3), 256, 0, pl->st, psi_of<A>(pl, s), pl->n3,
+                                   pl->scal + SC_SCALE, 0));
     pl->pending = false;
     pl->w_stage = ST_NONE;
   }
@@ -916,8 +919,8 @@ qfd_status period_launch(qfd_plan_t pl, int s, double* host) {
 template <class A>
 qfd_status finish_phase(qfd_plan_t pl, int s) {
   // leave the state normalised (its last finalised N2 is of the stored values)
-  QFD_RUN(PASS_OTHER, (k_scale<A><<<grid_for(pl->n3), 256, 0, pl->st>>>(psi_of<A>(pl, s), pl->n3, pl->scal + SC_N2, 1),
-                       cudaGetLastError()));
+  QFD_RUN(PASS_OTHER, pdl_launch(k_scale<A>, grid_for(pl->n3), 256, 0, pl->st, psi_of<A>(pl, s), pl->n3,
+                                 pl->scal + SC_N2, 1));
   pl->pending = false;
   pl->w_stage = ST_NONE;
   return QFD_OK;
@@ -1128,11 +1131,11 @@ qfd_status convert_state(qfd_plan_t pl, int s, int to_f32) {
   return with_policy(pl->arith16, [&](auto pol) -> qfd_status {
     using A = decltype(pol);
     if (to_f32) {
-      QFD_RUN(PASS_OTHER, (k_convert<A, F32><<<g, 256, 0, pl->st>>>(psi_of<A>(pl, s), psi_of<F32>(pl, s), pl->n3),
-                           cudaGetLastError()));
+      QFD_RUN(PASS_OTHER, pdl_launch(k_convert<A, F32>, g, 256, 0, pl->st, psi_of<A>(pl, s), psi_of<F32>(pl, s),
+                                     pl->n3));
     } else {
-      QFD_RUN(PASS_OTHER, (k_convert<F32, A><<<g, 256, 0, pl->st>>>(psi_of<F32>(pl, s), psi_of<A>(pl, s), pl->n3),
-                           cudaGetLastError()));
+      QFD_RUN(PASS_OTHER, pdl_launch(k_convert<F32, A>, g, 256, 0, pl->st, psi_of<F32>(pl, s), psi_of<A>(pl, s),
+                                     pl->n3));
     }
     if (pl->w_state == s) pl->w_stage = ST_NONE;
     return QFD_OK;
@@ -1668,10 +1671,10 @@ qfd_status qfd_set_psi(qfd_plan_t pl, int s, const double* psi, int on_device) {
     QFD_CK(cudaMemcpyAsync(pl->W, psi, bytes, kind, pl->st));
     if (pl->psi16)
       QFD_RUN(PASS_OTHER,
-              (k_convert<F64, DF><<<g, 256, 0, pl->st>>>(pl->W, psi_of<DF>(pl, s), pl->n3), cudaGetLastError()));
+              pdl_launch(k_convert<F64, DF>, g, 256, 0, pl->st, pl->W, psi_of<DF>(pl, s), pl->n3));
     else
       QFD_RUN(PASS_OTHER,
-              (k_convert<F64, F32><<<g, 256, 0, pl->st>>>(pl->W, psi_of<F32>(pl, s), pl->n3), cudaGetLastError()));
+              pdl_launch(k_convert<F64, F32>, g, 256, 0, pl->st, pl->W, psi_of<F32>(pl, s), pl->n3));
     pl->w_stage = ST_NONE;
   }
   if (pl->psi16 && pl->psi32 && (r = convert_state(pl, s, 1)) != QFD_OK) return r;
@@ -1687,13 +1690,13 @@ qfd_status qfd_fill_psi_uniform(qfd_plan_t pl, int s, uint64_t seed) {
   const int g = grid_for(pl->n3);
   if (pl->psi16 && pl->arith16 == 0)
     QFD_RUN(PASS_OTHER,
-            (k_fill_uniform<F64><<<g, 256, 0, pl->st>>>(psi_of<F64>(pl, s), pl->n3, seed), cudaGetLastError()));
+            pdl_launch(k_fill_uniform<F64>, g, 256, 0, pl->st, psi_of<F64>(pl, s), pl->n3, seed));
   if (pl->psi16 && pl->arith16 == 2)
     QFD_RUN(PASS_OTHER,
-            (k_fill_uniform<DF><<<g, 256, 0, pl->st>>>(psi_of<DF>(pl, s), pl->n3, seed), cudaGetLastError()));
+            pdl_launch(k_fill_uniform<DF>, g, 256, 0, pl->st, psi_of<DF>(pl, s), pl->n3, seed));
   if (pl->psi32)
     QFD_RUN(PASS_OTHER,
-            (k_fill_uniform<F32><<<g, 256, 0, pl->st>>>(psi_of<F32>(pl, s), pl->n3, seed), cudaGetLastError()));
+            pdl_launch(k_fill_uniform<F32>, g, 256, 0, pl->st, psi_of<F32>(pl, s), pl->n3, seed));
   pl->t[s] = 0;
   if (pl->w_state == s) pl->w_stage = ST_NONE;
   return QFD_OK;
@@ -1712,8 +1715,8 @@ qfd_status qfd_get_psi(qfd_plan_t pl, int s, double* out, int on_device) {
     if (A::id == 0) {
       QFD_CK(cudaMemcpyAsync(out, psi_of<A>(pl, s), bytes, kind, pl->st));
     } else {
-      QFD_RUN(PASS_OTHER, (k_convert<A, F64><<<grid_for(pl->n3), 256, 0, pl->st>>>(psi_of<A>(pl, s), pl->W, pl->n3),
-                           cudaGetLastError()));
+      QFD_RUN(PASS_OTHER, pdl_launch(k_convert<A, F64>, grid_for(pl->n3), 256, 0, pl->st, psi_of<A>(pl, s), pl->W,
+                                     pl->n3));
       pl->w_stage = ST_NONE;
       QFD_CK(cudaMemcpyAsync(out, pl->W, bytes, kind, pl->st));
     }
@@ -1736,8 +1739,8 @@ qfd_status qfd_observables(qfd_plan_t pl, int s, double min_sep_edge, double* ou
     using A = decltype(pol);
     qfd_status q = materialize<A>(pl, s);
     if (q != QFD_OK) return q;
-    QFD_RUN(PASS_OTHER, (k_observables<A><<<GS_BLOCKS, 256, 0, pl->st>>>(psi_of<A>(pl, s), lat, offgrid, half, pl->partG),
-                         cudaGetLastError()));
+    QFD_RUN(PASS_OTHER, pdl_launch(k_observables<A>, GS_BLOCKS, 256, 0, pl->st, psi_of<A>(pl, s), lat, offgrid,
+                                   half, pl->partG));
     return finalize(pl, pl->partG, NOBS, GS_BLOCKS, OP_OBS);
   });
   if (r != QFD_OK) return r;

@@ -33,6 +33,35 @@
 
 namespace qfd {
 
+// ================================================== programmatic launches
+// Every kernel of a step is launched with programmatic stream serialization:
+// its CTAs may be set up while the kernel before it drains, and pdl_begin, the
+// first statement of each, holds them until that kernel has completed and its
+// writes are visible.  Measured back to back on GB300 (small grids): 4.1 us a
+// launch without it, 1.4-1.7 us with it.  No kernel releases its successor early
+// (griddepcontrol.launch_dependents): the waiting CTAs then pile up on the SMs
+// that drain first and leave the others idle (96^3 double-float step 77 -> 101 us).
+// Arrays that an earlier kernel of the stream may have written are read through
+// plain pointers (no const __restrict__: the read-only path is not ordered by
+// the wait, and the compiler may move such loads above it).
+__device__ __forceinline__ void pdl_begin() {
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+}
+template <class... P, class... A>
+cudaError_t pdl_launch(void (*kern)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, A&&... args) {
+  cudaLaunchAttribute at{};
+  at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at.val.programmaticStreamSerializationAllowed = 1;
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = grid;
+  cfg.blockDim = block;
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = st;
+  cfg.attrs = &at;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, kern, static_cast<P>(args)...);
+}
+
 // ============================================================ float/double
 template <typename C> __device__ __forceinline__ C cadd(C a, C b) { return C{a.x + b.x, a.y + b.y}; }
 template <typename C> __device__ __forceinline__ C csub(C a, C b) { return C{a.x - b.x, a.y - b.y}; }
@@ -1002,13 +1031,24 @@ template <typename C, int PS, int T> struct AccLine {
 #ifndef QFD_LINE_TARGET8
 #define QFD_LINE_TARGET8 128
 #endif
-// Resident CTAs per SM asked of the compiler for the complex128 kernels: 1024
-// threads (64 registers each).  The fixed-point transforms are chains of integer
-// operations, bound by how many warps hide their latency: at 512^3 with 512 /
-// 768 / 1024 threads an SM the y pass takes 1.49 / 1.32 / 1.26 ms, the z pass
-// 3.20 / 2.82 / 2.58 and pass A 4.54 / 3.98 / 3.76 (at most 32 bytes spilled).
-__host__ __device__ constexpr int f64_ctas(int threads) {
-  return 1024 / threads < 1 ? 1 : (1024 / threads > 8 ? 8 : 1024 / threads);
+// Resident CTAs per SM asked of the compiler, as threads per SM (registers are
+// 65536 over them).  Complex128 asks for 1024 everywhere: the fixed-point
+// transforms are chains of integer operations, bound by how many warps hide
+// their latency; at 512^3 with 512 / 768 / 1024 threads an SM the y pass takes
+// 1.49 / 1.32 / 1.26 ms, the z pass 3.20 / 2.82 / 2.58 and pass A 4.54 / 3.98 /
+// 3.76 (at most 32 bytes spilled).  The other two keep what their transforms
+// need without spilling; without a bound the compiler takes up to twice that
+// behind the wait of pdl_begin (double-float z pass 2.60 -> 3.33 ms).
+__host__ __device__ constexpr int ctas(int threads, int resident) {
+  return resident / threads < 1 ? 1 : (resident / threads > 8 ? 8 : resident / threads);
+}
+template <class A, int N, int ZG, int R> constexpr int z_resident() {
+  if (A::id == 0) return ZG == 1 ? 1024 : 1;
+  if (A::id == 2) return ZG > 1 ? 1 : N % 3 == 0 ? 512 : N <= 64 ? 1024 : 768;
+  return R == 1 ? 384 : N % 3 == 0 || (ZG > 1 && N >= 512) ? 512 : ZG == 1 ? 768 : 640;
+}
+template <class A, int N, bool LOWER> constexpr int project_resident() {
+  return A::id == 1 || (A::id == 0 && !LOWER) ? 1024 : A::id == 2 && !LOWER && N % 3 != 0 && N <= 256 ? 768 : 512;
 }
 template <int N, int CMIN> struct TileCols {
   static constexpr int T = N / FftPlan<N>::E;
@@ -1259,13 +1299,14 @@ __device__ __forceinline__ void fft_strided_body(typename A::C* W, const typenam
 // many warps in flight), the 16-byte arithmetics take what their registers allow.
 template <class A, int N, int YC> struct YOcc {
   static constexpr int THREADS = N / FftPlan<N>::E * YC;
-  static constexpr int B0 = A::id == 1 ? 1536 / THREADS : A::id == 0 ? f64_ctas(THREADS) : 1;
+  static constexpr int B0 = A::id == 1 ? 1536 / THREADS : A::id == 0 ? ctas(THREADS, 1024) : 1;
   static constexpr int value = B0 < 1 ? 1 : (B0 > 8 ? 8 : B0);
 };
 template <class A, int N, int DIR, int YC, int R = 0>
 __global__ void __launch_bounds__(FftPlan<N, R>::T * YC, R == 0 ? YOcc<A, N, YC>::value : 1)
 k_fft_strided(const __grid_constant__ BatchY b, int64_t stride, int tiles_inner, int64_t outer_stride) {
   using C = typename A::C;
+  pdl_begin();
   fft_strided_body<A, N, DIR, YC, R>(static_cast<C*>(b.W[blockIdx.y]), static_cast<const C*>(b.tw[blockIdx.y]),
                                      stride, tiles_inner, outer_stride);
 }
@@ -1331,8 +1372,9 @@ template <class A, int N, int R> struct ZLines {
 };
 template <class A, int N, bool PARSEVAL, int ZG, int R = 0>
 __global__ void __launch_bounds__(FftPlan<N, R>::T * ZLines<A, N, R>::value,
-                                  A::id == 0 && ZG == 1 ? f64_ctas(FftPlan<N, R>::T * ZLines<A, N, R>::value) : 1)
+                                  ctas(FftPlan<N, R>::T * ZLines<A, N, R>::value, z_resident<A, N, ZG, R>()))
 k_zpass(const __grid_constant__ BatchZ b) {
+  pdl_begin();
   using C = typename A::C;
   const int i = blockIdx.y;
   zpass_body<A, N, PARSEVAL, ZG, R, ZLines<A, N, R>::value>(static_cast<C*>(b.W[i]), static_cast<const C*>(b.tw[i]),
@@ -1353,8 +1395,8 @@ __device__ __forceinline__ void update_x_core(typename A::C (&v)[FftPlan<N>::E],
                                               const typename A::U (&cf)[FftPlan<N>::E], int t, int col, int64_t base,
                                               typename A::C* W, typename A::C* __restrict__ psi,
                                               const typename A::U* __restrict__ uin, const UpdParams& upar,
-                                              const typename A::VT* __restrict__ V, const double* __restrict__ scale,
-                                              const float* __restrict__ scale_f, const typename A::C* __restrict__ tw,
+                                              const typename A::VT* __restrict__ V, const double* scale,
+                                              const float* scale_f, const typename A::C* __restrict__ tw,
                                               typename A::C* sm, typename A::Acc& nacc, typename A::Full& facc) {
   using C = typename A::C;
   using SH = Shape<A, N>;
@@ -1388,8 +1430,8 @@ __device__ __forceinline__ void update_x_core(typename A::C (&v)[FftPlan<N>::E],
 template <class A, int N, int STATS, int XC>
 __device__ __forceinline__ void update_x_body(typename A::C* W, typename A::C* __restrict__ psi,
                                               const typename A::U* __restrict__ uin, const UpdParams& upar,
-                                              const typename A::VT* __restrict__ V, const double* __restrict__ scale,
-                                              const float* __restrict__ scale_f, const typename A::C* __restrict__ tw,
+                                              const typename A::VT* __restrict__ V, const double* scale,
+                                              const float* scale_f, const typename A::C* __restrict__ tw,
                                               double* __restrict__ part) {
   using C = typename A::C;
   using U = typename A::U;
@@ -1420,8 +1462,9 @@ __device__ __forceinline__ void update_x_body(typename A::C* W, typename A::C* _
 // resident CTAs per SM.
 template <class A, int N, int STATS, int XC>
 __global__ void __launch_bounds__(N / FftPlan<N>::E * XC,
-                                  A::id == 0 ? f64_ctas(N / FftPlan<N>::E * XC) : XC < Shape<A, N>::XCOLS ? 2 : 1)
+                                  A::id == 0 ? ctas(N / FftPlan<N>::E * XC, 1024) : XC < Shape<A, N>::XCOLS ? 2 : 1)
 k_update_x(const __grid_constant__ BatchU b, uint32_t scaled) {
+  pdl_begin();
   using C = typename A::C;
   const int i = blockIdx.y;
   update_x_body<A, N, STATS, XC>(static_cast<C*>(b.W[i]), static_cast<C*>(b.psi[i]),
@@ -1434,10 +1477,11 @@ k_update_x(const __grid_constant__ BatchU b, uint32_t scaled) {
 // psi_out) into W; partials per STATS of the scaled input.  src may alias W
 // (each CTA reads its whole tile before writing it).
 template <class A, int N, int STATS>
-__global__ void __launch_bounds__(Shape<A, N>::XTHREADS, A::id == 0 ? f64_ctas(Shape<A, N>::XTHREADS) : 1)
+__global__ void __launch_bounds__(Shape<A, N>::XTHREADS, ctas(Shape<A, N>::XTHREADS, 1024))
 k_forward_x(const typename A::C* src, typename A::C* W, typename A::C* psi_out, const typename A::VT* __restrict__ V,
-            const double* __restrict__ scale, const float* __restrict__ scale_f, const typename A::C* __restrict__ tw,
+            const double* scale, const float* scale_f, const typename A::C* __restrict__ tw,
             double* __restrict__ part) {
+  pdl_begin();
   using C = typename A::C;
   using SH = Shape<A, N>;
   extern __shared__ __align__(16) unsigned char smraw[];
@@ -1494,8 +1538,9 @@ __device__ __forceinline__ int reflect1(int x, int offgrid) {
 // accumulator and stored as FP64 partials (2 per lower state).
 template <class A, int N>
 __global__ void __launch_bounds__(256)
-k_gs_dots(const typename A::C* __restrict__ psi, LowerPtrs lower, int k, int parity, int offgrid,
+k_gs_dots(const typename A::C* psi, LowerPtrs lower, int k, int parity, int offgrid,
           double* __restrict__ part) {
+  pdl_begin();
   using C = typename A::C;
   constexpr int64_t N3 = (int64_t)N * N * N;
   typename A::Dot acc[MAX_LOWER];
@@ -1529,11 +1574,12 @@ k_gs_dots(const typename A::C* __restrict__ psi, LowerPtrs lower, int k, int par
 // LOWER: whether there are lower states (k > 0); the parity-only instance
 // carries no Gram-Schmidt code at all.
 template <class A, int N, int STATS, bool LOWER = true>
-__global__ void __launch_bounds__(Shape<A, N>::XTHREADS, A::id == 0 && !LOWER ? f64_ctas(Shape<A, N>::XTHREADS) : 1)
-k_project_x(const typename A::C* __restrict__ src, LowerPtrs lower, const double* __restrict__ sums, int k, int parity,
-            int offgrid, typename A::C* __restrict__ dst, typename A::C* __restrict__ W,
+__global__ void __launch_bounds__(Shape<A, N>::XTHREADS, ctas(Shape<A, N>::XTHREADS, project_resident<A, N, LOWER>()))
+k_project_x(const typename A::C* src, LowerPtrs lower, const double* sums, int k, int parity,
+            int offgrid, typename A::C* dst, typename A::C* W,
             const typename A::VT* __restrict__ V,
             const typename A::C* __restrict__ tw, double* __restrict__ part) {
+  pdl_begin();
   using C = typename A::C;
   using SH = Shape<A, N>;
   extern __shared__ __align__(16) unsigned char smraw[];
@@ -1587,7 +1633,8 @@ k_project_x(const typename A::C* __restrict__ src, LowerPtrs lower, const double
 
 // psi *= f in the policy's arithmetic, f = scal[0] (mode 0) or 1 / sqrt(scal[1]) (mode 1).
 template <class A>
-__global__ void k_scale(typename A::C* __restrict__ psi, int64_t n3, const double* __restrict__ f_or_n2, int mode) {
+__global__ void k_scale(typename A::C* psi, int64_t n3, const double* f_or_n2, int mode) {
+  pdl_begin();
   const double f = mode == 0 ? f_or_n2[0] : 1.0 / sqrt(f_or_n2[0]);
   const typename A::S fs = A::scalar(f);
   for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n3; i += (int64_t)gridDim.x * blockDim.x)
@@ -1596,8 +1643,9 @@ __global__ void k_scale(typename A::C* __restrict__ psi, int64_t n3, const doubl
 
 // dst = src * f, f = *scale (1 when scale is null), in the policy's arithmetic.
 template <class A>
-__global__ void k_scale_copy(typename A::C* __restrict__ dst, const typename A::C* __restrict__ src, int64_t n3,
-                             const double* __restrict__ scale) {
+__global__ void k_scale_copy(typename A::C* dst, const typename A::C* src, int64_t n3,
+                             const double* scale) {
+  pdl_begin();
   const typename A::S fs = A::scalar(scale ? scale[0] : 1.0);
   for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n3; i += (int64_t)gridDim.x * blockDim.x)
     dst[i] = cscale(src[i], fs);

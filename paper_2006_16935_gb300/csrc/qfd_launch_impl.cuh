@@ -47,8 +47,8 @@ cudaError_t Launch<A, N>::forward_x(const LaunchArgs& a, int* nblocks) {
   const int grid = (int)((int64_t)N * N / SH::XCOLS);
   auto go = [&](auto kern) {
     ensure_smem(kern, smem);
-    kern<<<grid, SH::XTHREADS, smem, a.stream>>>((const C*)a.src, (C*)a.W, (C*)a.psi_out, (const VT*)a.V, a.scale,
-                                                  a.scale_f, (const C*)a.tw, a.part);
+    pdl_launch(kern, grid, SH::XTHREADS, smem, a.stream, (const C*)a.src, (C*)a.W, (C*)a.psi_out, (const VT*)a.V,
+               a.scale, a.scale_f, (const C*)a.tw, a.part);
   };
   if (a.stats == STATS_FULL) go(k_forward_x<A, N, STATS_FULL>);
   else if (a.stats == STATS_NORM) go(k_forward_x<A, N, STATS_NORM>);
@@ -87,8 +87,8 @@ cudaError_t Launch<A, N>::project_x(const LaunchArgs& a, int* nblocks) {
   for (int j = 0; j < MAX_LOWER; ++j) lp.p[j] = a.lower[j];
   auto go = [&](auto kern) {
     ensure_smem(kern, smem);
-    kern<<<grid, SH::XTHREADS, smem, a.stream>>>((const C*)a.src, lp, a.sums, a.k, a.parity, a.offgrid,
-                                                      (C*)a.dst, (C*)a.W, (const VT*)a.V, (const C*)a.tw, a.part);
+    pdl_launch(kern, grid, SH::XTHREADS, smem, a.stream, (const C*)a.src, lp, a.sums, a.k, a.parity, a.offgrid,
+               (C*)a.dst, (C*)a.W, (const VT*)a.V, (const C*)a.tw, a.part);
   };
   if (a.k > 0) {
     if (a.stats == STATS_FULL) go(k_project_x<A, N, STATS_FULL, true>);
@@ -105,8 +105,8 @@ template <class A, int N>
 cudaError_t Launch<A, N>::gs_dots(const LaunchArgs& a, int nblocks) {
   LowerPtrs lp;
   for (int j = 0; j < MAX_LOWER; ++j) lp.p[j] = a.lower[j];
-  k_gs_dots<A, N><<<nblocks, 256, 0, a.stream>>>((const typename A::C*)a.src, lp, a.k, a.parity, a.offgrid, a.part);
-  return cudaGetLastError();
+  return pdl_launch(k_gs_dots<A, N>, nblocks, 256, 0, a.stream, (const typename A::C*)a.src, lp, a.k, a.parity,
+                    a.offgrid, a.part);
 }
 
 template <class A, int N>
@@ -117,8 +117,8 @@ cudaError_t Launch<A, N>::fft_y_batch(const BatchY& b, int count, int dir, int v
     const size_t smem = (size_t)N * yc * sizeof(C);
     const int tiles_inner = N / yc;
     ensure_smem(kern, smem);
-    kern<<<dim3(N * tiles_inner, count), tpc * yc, smem, st>>>(b, (int64_t)N, tiles_inner,
-                                                                          (int64_t)N * N);
+    pdl_launch(kern, dim3(N * tiles_inner, count), tpc * yc, smem, st, b, (int64_t)N, tiles_inner,
+               (int64_t)N * N);
   };
   if constexpr (SH::HAS_R1) {
     if (vy == 2) {  // the two-stage radix schedule
@@ -148,7 +148,7 @@ cudaError_t Launch<A, N>::zpass_batch(const BatchZ& b, int count, int parseval, 
       const int grid = (int)((int64_t)N * N / SH::LINES_R1);
       auto go1 = [&](auto kern) {
         ensure_smem(kern, smem);
-        kern<<<dim3(grid, count), SH::T1 * SH::LINES_R1, smem, st>>>(b);
+        pdl_launch(kern, dim3(grid, count), SH::T1 * SH::LINES_R1, smem, st, b);
       };
       if (parseval) go1(k_zpass<A, N, true, 1, 1>);
       else go1(k_zpass<A, N, false, 1, 1>);
@@ -162,7 +162,7 @@ cudaError_t Launch<A, N>::zpass_batch(const BatchZ& b, int count, int parseval, 
   const int grid = (int)((int64_t)N * N / (SH::LINES * zg));
   auto go = [&](auto kern) {
     ensure_smem(kern, smem);
-    kern<<<dim3(grid, count), SH::LINE_THREADS, smem, st>>>(b);
+    pdl_launch(kern, dim3(grid, count), SH::LINE_THREADS, smem, st, b);
   };
   if (zg == 1) {
     if (parseval) go(k_zpass<A, N, true, 1>);
@@ -195,7 +195,7 @@ cudaError_t Launch<A, N>::update_x_batch(const BatchU& b, int count, uint32_t sc
       const int grid = sms < NT ? sms : NT;
       auto go = [&](auto kern) {
         cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)TS::SMEM);
-        kern<<<dim3(grid, count), TS::THREADS, TS::SMEM, st>>>(b, scaled, tma_test);
+        pdl_launch(kern, dim3(grid, count), TS::THREADS, TS::SMEM, st, b, scaled, tma_test);
       };
       if (stats == STATS_FULL) go(k_update_x_tma<A, N, STATS_FULL>);
       else if (stats == STATS_NORM) go(k_update_x_tma<A, N, STATS_NORM>);
@@ -208,7 +208,7 @@ cudaError_t Launch<A, N>::update_x_batch(const BatchU& b, int count, uint32_t sc
     const size_t smem = (size_t)N * xc * sizeof(C);
     const int grid = (int)((int64_t)N * N / xc);
     ensure_smem(kern, smem);
-    kern<<<dim3(grid, count), SH::T * xc, smem, st>>>(b, scaled);
+    pdl_launch(kern, dim3(grid, count), SH::T * xc, smem, st, b, scaled);
     if (nblocks) *nblocks = grid;
   };
   if (vx == 1) {

@@ -99,6 +99,7 @@ template <class A, int N> struct TmaShape {
 template <class A, int N, int STATS>
 __global__ void __launch_bounds__(TmaShape<A, N>::THREADS, 1)
 k_update_x_tma(const __grid_constant__ BatchU b, uint32_t scaled, int test_skip) {
+  pdl_begin();
   using C = typename A::C;
   using U = typename A::U;
   using TS = TmaShape<A, N>;
