@@ -312,6 +312,10 @@ qfd_status qfd_autotune(qfd_plan_t plan, double* ms_out);
  * persistent pass A.  The two-stage schedule exists for complex64 at
  * n = 128..1024 and the TMA pass A for complex64 at n = 256..1024 (when the
  * plan could build its tensor maps, qfd_has_tma); elsewhere 2 runs the default.
+ * With y_variant 0 and z_variant -1 (the defaults) the y and z passes of small
+ * lattices (complex64 up to n = 128, 16-byte arithmetics up to 32) run as one
+ * launch over the planes x = const; any other setting, and the per-pass
+ * timing of qfd_timing_enable, runs them separately.
  *
  * The TMA-staged pass A runs one persistent CTA per SM; the Tensor Memory
  * Accelerator copies the next tile's W, psi and V (2D tensor maps of the

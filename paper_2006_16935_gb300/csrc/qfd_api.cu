@@ -661,9 +661,28 @@ qfd_status pass_forward_x(qfd_plan_t pl, const void* src, void* psi_out, bool us
   return QFD_OK;
 }
 
+// Whether the plan's passes B, C and D run as one launch over planes: with the
+// default launch shapes, where the launcher has it (PlaneShape).  Hand-set or
+// tuned shapes of the y and z passes select the separate passes, and so does
+// the per-pass timing, which reports each of them.
+template <class A> bool plane_path(qfd_plan_t pl) {
+  return !pl->timing && pl->tune_vy[A::id] == 0 && pl->tune_vz[A::id] == -1 && has_plane<A>(pl->p.n);
+}
+
+// Runs the rest of passes B, C and D.  With parseval_at_c the Parseval partials
+// are left in partC and the separate passes stop before pass D.
 template <class A>
 qfd_status advance_to_d(qfd_plan_t pl, int parseval_at_c) {
   LaunchArgs a = base_args<A>(pl);
+  if (pl->w_stage == ST_X && plane_path<A>(pl)) {
+    a.part = pl->partC;
+    a.stats = parseval_at_c;
+    int nb = 0;
+    QFD_RUN(PASS_ZKIN, launch_plane<A>(a, &nb));
+    pl->nC = nb;
+    pl->w_stage = ST_D;
+    return QFD_OK;
+  }
   if (pl->w_stage == ST_X) {
     QFD_RUN(PASS_FWD_Y, launch_fft_y<A>(a, -1));
     pl->w_stage = ST_XY;
@@ -1120,8 +1139,20 @@ qfd_status autotune_policy(qfd_plan_t pl, double* ms) {
     }
     pl->tune_vx[A::id] = argmin(ms + 6, nxv);
   }
-  pl->tune_vy[A::id] = argmin(ms, nv);
-  pl->tune_vz[A::id] = argmin(ms + 3, nv);
+  const int by = argmin(ms, nv), bz = argmin(ms + 3, nv);
+  pl->tune_vy[A::id] = by;
+  pl->tune_vz[A::id] = bz;
+  if (has_plane<A>(pl->p.n)) {  // the default shapes: passes B, C and D in one launch
+    LaunchArgs a = base_args<A>(pl);
+    a.part = pl->partC;
+    a.stats = 0;
+    double mp = INFINITY;
+    if ((r = time_launch(pl, [&]() { return launch_plane<A>(a, nullptr); }, 2, 5, &mp)) != QFD_OK) return r;
+    if (mp < 2.0 * ms[by] + ms[3 + bz]) {
+      pl->tune_vy[A::id] = 0;
+      pl->tune_vz[A::id] = -1;
+    }
+  }
   return QFD_OK;
 }
 
@@ -1234,9 +1265,13 @@ qfd_status batch_step_once(qfd_plan_s* const* pls, const int* ss, int count, int
   }
   if (nx > 0) {
     qfd_plan_t pl = p0;  // the batched launches are counted and timed on plans[0]
-    QFD_RUN(PASS_FWD_Y, launch_fft_y_batch<A>(n, by, nx, -1, vy, st));
-    QFD_RUN(PASS_ZKIN, launch_zpass_batch<A>(n, bz, nx, 0, vz, st, nullptr));
-    QFD_RUN(PASS_INV_Y, launch_fft_y_batch<A>(n, by, nx, +1, vy, st));
+    if (plane_path<A>(p0)) {
+      QFD_RUN(PASS_ZKIN, launch_plane_batch<A>(n, bz, nx, 0, st, nullptr));
+    } else {
+      QFD_RUN(PASS_FWD_Y, launch_fft_y_batch<A>(n, by, nx, -1, vy, st));
+      QFD_RUN(PASS_ZKIN, launch_zpass_batch<A>(n, bz, nx, 0, vz, st, nullptr));
+      QFD_RUN(PASS_INV_Y, launch_fft_y_batch<A>(n, by, nx, +1, vy, st));
+    }
   }
   // pass A, grouped by partial-sum mode as step_once chooses it: STATS_NORM
   // where the step ends in a cadence without a projection, STATS_FULL on the
@@ -1339,13 +1374,17 @@ qfd_status batch_period_launch(qfd_plan_s* const* pls, const int* ss, int count,
   {
     qfd_plan_t pl = p0;
     const int vy = p0->tune_vy[A::id], vz = p0->tune_vz[A::id];
-    QFD_RUN(PASS_FWD_Y, launch_fft_y_batch<A>(n, by, count, -1, vy, st));
-    QFD_RUN(PASS_ZKIN, launch_zpass_batch<A>(n, bz, count, 1, vz, st, &nc));
+    if (plane_path<A>(p0)) {
+      QFD_RUN(PASS_ZKIN, launch_plane_batch<A>(n, bz, count, 1, st, &nc));
+    } else {
+      QFD_RUN(PASS_FWD_Y, launch_fft_y_batch<A>(n, by, count, -1, vy, st));
+      QFD_RUN(PASS_ZKIN, launch_zpass_batch<A>(n, bz, count, 1, vz, st, &nc));
+    }
   }
   for (int i = 0; i < count; ++i) {
     qfd_plan_t pl = pls[i];
     pl->nC = nc;
-    pl->w_stage = ST_C;
+    pl->w_stage = plane_path<A>(p0) ? ST_D : ST_C;
     if ((r = finalize(pl, pl->partC, 1, pl->nC, OP_ENERGY)) != QFD_OK) return r;
     QFD_CK(cudaMemcpyAsync(pl->hscal, pl->scal, SC_COUNT * sizeof(double), cudaMemcpyDeviceToHost, st));
     QFD_CK(cudaMemcpyAsync(pl->hscal + SC_COUNT, pl->errflag, sizeof(int), cudaMemcpyDeviceToHost, st));

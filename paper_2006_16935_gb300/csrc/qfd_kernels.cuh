@@ -918,7 +918,7 @@ __device__ __forceinline__ void fft_line(typename A::C (&v)[FftPlan<N, R>::E], i
 }
 
 // Shared-memory views. Tile of CW columns of a strided axis: [pos][col] with a
-// row pitch of PITCH >= CW elements.  (Rows of 64 bytes take twice the
+// row pitch of PITCH >= CW elements (off: where the column sits in a row).  (Rows of 64 bytes take twice the
 // minimum shared-memory wavefronts in the first exchange, where each thread
 // writes its E outputs E rows apart; a padding row every E rows removes that
 // but was measured slower at 512^3, by the index arithmetic it adds to every
@@ -927,19 +927,20 @@ __device__ __forceinline__ void fft_line(typename A::C (&v)[FftPlan<N, R>::E], i
 // line_max (complex128): reduces mx over the threads of a line and returns
 // whether any line that shares the tile's barriers is `odd`.  The partial
 // maxima go to one of two buffers in turn, so that one barrier suffices.
-template <typename C, int CW, int T> struct AccTile {
+template <typename C, int CW, int T, int PITCH = CW> struct AccTile {
   static constexpr int G = CW >= 32 ? 1 : (32 / CW < T ? 32 / CW : T);  // threads of a column in a warp
   static constexpr int ROWS = T / G;                                       // partial maxima of a column
   static constexpr int MAXN = 2 * ROWS * CW;
   C* sm;
-  int col;
+  int off, col;
   int* mxs;
   int flip;
-  __device__ __forceinline__ AccTile(C* s, int c, int* m = nullptr, int f = 0) : sm(s), col(c), mxs(m), flip(f) {}
-  template <typename D> __device__ __forceinline__ AccTile<D, CW, T> as() const {
-    return AccTile<D, CW, T>(reinterpret_cast<D*>(sm), col);
+  __device__ __forceinline__ AccTile(C* s, int o, int c, int* m = nullptr)
+      : sm(s), off(o), col(c), mxs(m), flip(0) {}
+  template <typename D> __device__ __forceinline__ AccTile<D, CW, T, PITCH> as() const {
+    return AccTile<D, CW, T, PITCH>(reinterpret_cast<D*>(sm), off, col);
   }
-  __device__ __forceinline__ C& at(int pos) { return sm[pos * CW + col]; }
+  __device__ __forceinline__ C& at(int pos) { return sm[pos * PITCH + off]; }
   __device__ __forceinline__ void sync() { __syncthreads(); }
   __device__ __forceinline__ bool line_max(int& mx, bool odd, int t) {
 #pragma unroll
@@ -982,7 +983,7 @@ template <typename C, int PS, int T> struct AccLine {
     if constexpr (T <= 32) {
 #pragma unroll
       for (int o = 1; o < T; o <<= 1) mx = max(mx, __shfl_xor_sync(0xffffffffu, mx, o));
-      return __any_sync(0xffffffffu, odd);
+      return __any_sync(__activemask(), odd);
     } else {
       if (odd) mx = 0x7fffffff;
       mx = __reduce_max_sync(0xffffffffu, mx);
@@ -1286,7 +1287,7 @@ __device__ __forceinline__ void fft_strided_body(typename A::C* W, const typenam
   for (int m = 0; m < PL::E; ++m) v[m] = W[base + (int64_t)(t + m * PL::T) * stride];
   using AT = AccTile<C, YC, PL::T>;
   __shared__ int mxs[A::id == 0 ? AT::MAXN : 1];
-  AT acc{sm, col, mxs};
+  AT acc{sm, col, col, mxs};
   // complex64 inverse y pass and the two-stage schedule: computed twiddles
   // (measured faster there; the forward y pass of schedule 0 is faster with
   // the table)
@@ -1382,6 +1383,96 @@ k_zpass(const __grid_constant__ BatchZ b) {
                                                              b.part[i]);
 }
 
+// Passes B, C and D in one launch where a plane x = const fits in shared memory
+// (a step touches y and z only inside such a plane): one CTA per plane reads
+// it once, transforms along y and z, multiplies by T(k)/N^3, transforms back
+// and writes it once.  16 instead of 48 bytes a site (complex64) and two
+// launches a step instead of four.  The plane sits in shared memory as rows of
+// one y with the z lines' padding, and the y transforms exchange in that same
+// layout, so the two directions share the buffer and nothing is copied.
+// Measured us a step, separate passes then this one: complex64 16^3 6.95 and 3.92,
+// 64^3 9.85 and 7.41, 96^3 22.3 and 20.8, 128^3 33.1 and 29.8; complex128 32^3
+// 24.4 and 19.6, 64^3 31.0 and 39.9; double-float 32^3 15.4 and 13.5, 64^3 19.7
+// and 23.2 (the last of each pair is why the line is drawn at 32).  Each thread owns one radix column (E elements) of the plane, or GRP of them
+// in turn where the plane has more than 1024.
+template <class A, int N> struct PlaneShape {
+  static constexpr int T = N / FftPlan<N>::E;
+  static constexpr size_t SMEM = (size_t)N * Shape<A, N>::LPAD * sizeof(typename A::C);
+  // 8-byte sites: up to 128 (139 KB).  16-byte sites: up to 32; above that the
+  // passes are bound by arithmetic, and N CTAs do not fill the SMs.
+  static constexpr bool OK = N <= (sizeof(typename A::C) == 8 ? 128 : 32);
+  static constexpr int GRP = T * N > 1024 ? T * N / 1024 : 1;
+  static constexpr int COLS = N / GRP;          // columns (and lines) at a time
+  static constexpr int THREADS = T * COLS;
+};
+template <class A, int N, bool PARSEVAL>
+__global__ void __launch_bounds__(PlaneShape<A, N>::THREADS, ctas(PlaneShape<A, N>::THREADS, 1024))
+k_plane(const __grid_constant__ BatchZ b) {
+  pdl_begin();
+  using C = typename A::C;
+  using T = typename A::T;
+  using SH = Shape<A, N>;
+  using PS = PlaneShape<A, N>;
+  using AT = AccTile<C, PS::COLS, PS::T, SH::LPAD>;
+  using AL = AccLine<C, SH::PAD_SHIFT, PS::T>;
+  constexpr int E = FftPlan<N>::E, TT = PS::T;
+  extern __shared__ __align__(16) unsigned char smraw[];
+  C* sm = reinterpret_cast<C*>(smraw);
+  __shared__ int mxs[A::id == 0 ? AT::MAXN : 1];
+  const int lat = blockIdx.y, x = blockIdx.x;
+  C* W = static_cast<C*>(b.W[lat]) + (int64_t)x * N * N;
+  const C* tw = static_cast<const C*>(b.tw[lat]);
+  const T* ktab = static_cast<const T*>(b.ktab[lat]);
+  const KinParams& kp = b.kp[lat];
+  typename A::Pars pacc;
+  const int col0 = threadIdx.x % PS::COLS, ty = threadIdx.x / PS::COLS;  // y transforms: column z, thread of it
+  const int l0 = threadIdx.x / TT, tz = threadIdx.x % TT;                // z transforms: line y, thread of it
+  C v[E];
+#pragma unroll
+  for (int g = 0; g < PS::GRP; ++g) {
+    const int col = col0 + g * PS::COLS;
+    AT acc{sm, col + (col >> SH::PAD_SHIFT), col0, mxs};
+#pragma unroll
+    for (int m = 0; m < E; ++m) v[m] = W[(ty + m * TT) * N + col];
+    fft_line<A, N, -1>(v, ty, tw, acc);
+#pragma unroll
+    for (int m = 0; m < E; ++m) acc.at(ty + m * TT) = v[m];
+  }
+  __syncthreads();
+#pragma unroll
+  for (int g = 0; g < PS::GRP; ++g) {
+    const int l = l0 + g * PS::COLS;
+    AL acc{sm + l * SH::LPAD, l0};
+#pragma unroll
+    for (int m = 0; m < E; ++m) v[m] = acc.at(tz + m * TT);
+    acc.sync();
+    fft_line<A, N, -1, AL, true>(v, tz, tw, acc);
+    const T sxy = A::kadd(ktab[x], ktab[l]);
+#pragma unroll
+    for (int m = 0; m < E; ++m) {
+      const T tk = A::kin(A::kadd(sxy, ktab[tz + m * TT]), kp);
+      if constexpr (PARSEVAL) pacc.add(tk, v[m]);
+      v[m] = cscale(v[m], tk);
+    }
+    fft_line<A, N, +1, AL, true>(v, tz, tw, acc);
+#pragma unroll
+    for (int m = 0; m < E; ++m) acc.at(tz + m * TT) = v[m];
+  }
+  __syncthreads();
+#pragma unroll
+  for (int g = 0; g < PS::GRP; ++g) {
+    const int col = col0 + g * PS::COLS;
+    AT acc{sm, col + (col >> SH::PAD_SHIFT), col0, mxs};
+#pragma unroll
+    for (int m = 0; m < E; ++m) v[m] = acc.at(ty + m * TT);
+    acc.sync();
+    fft_line<A, N, +1, AT, true>(v, ty, tw, acc);
+#pragma unroll
+    for (int m = 0; m < E; ++m) W[(ty + m * TT) * N + col] = v[m];
+  }
+  if constexpr (PARSEVAL) pars_store<A>(pacc, b.part[lat]);
+}
+
 // Pass A: inverse DFT_x of W gives H_K psi at the tile's sites; the update of
 // Eq. (iter_proced) with the coefficients of Sec. 2.2 (read precomputed for
 // complex128, derived from V in the FP32-pipe arithmetics), times an optional
@@ -1403,7 +1494,7 @@ __device__ __forceinline__ void update_x_core(typename A::C (&v)[FftPlan<N>::E],
   constexpr int64_t S = (int64_t)N * N;
   using AT = AccTile<C, XC, SH::T>;
   __shared__ int mxs[A::id == 0 ? AT::MAXN : 1];
-  AT acc{sm, col, mxs};
+  AT acc{sm, col, col, mxs};
   fft_line<A, N, +1>(v, t, tw, acc);
   const bool scaled = scale != nullptr;
   typename A::S s{};
@@ -1510,7 +1601,7 @@ k_forward_x(const typename A::C* src, typename A::C* W, typename A::C* psi_out, 
   }
   using AT = AccTile<C, SH::XCOLS, SH::T>;
   __shared__ int mxs[A::id == 0 ? AT::MAXN : 1];
-  AT acc{sm, col, mxs};
+  AT acc{sm, col, col, mxs};
   fft_line<A, N, -1>(v, t, tw, acc);
 #pragma unroll
   for (int m = 0; m < SH::E; ++m) W[base + (t + m * SH::T) * S] = v[m];
@@ -1623,7 +1714,7 @@ k_project_x(const typename A::C* src, LowerPtrs lower, const double* sums, int k
   }
   using AT = AccTile<C, SH::XCOLS, SH::T>;
   __shared__ int mxs[A::id == 0 ? AT::MAXN : 1];
-  AT acc{sm, col, mxs};
+  AT acc{sm, col, col, mxs};
   fft_line<A, N, -1>(v, t, tw, acc);
 #pragma unroll
   for (int m = 0; m < SH::E; ++m) W[base + (t + m * SH::T) * S] = v[m];

@@ -159,6 +159,12 @@ template <class A, int N> struct Launch {
   static cudaError_t zpass_batch(const BatchZ& b, int count, int parseval, int vz, cudaStream_t st, int* nblocks);
   static cudaError_t update_x_batch(const BatchU& b, int count, uint32_t scaled, int stats, int vx, cudaStream_t st,
                                     int* nblocks, int tma_test = 0);
+  // passes B, C and D of `count` lattices as one launch over their planes, with
+  // or without the Parseval partial (where has_plane(): the plane fits in
+  // shared memory)
+  static cudaError_t plane_batch(const BatchZ& b, int count, int parseval, cudaStream_t st, int* nblocks);
+  static cudaError_t plane(const LaunchArgs& a, int* nblocks);
+  static bool has_plane();
   static int tma_xt();  // tile width of the TMA-staged pass A (vx = 2), 0 where it does not exist
 };
 
@@ -216,6 +222,21 @@ cudaError_t launch_update_x_batch(int64_t n, const BatchU& b, int count, uint32_
   return dispatch_n(n, [&](auto t) {
     return Launch<A, decltype(t)::value>::update_x_batch(b, count, scaled, stats, vx, st, nb, tma_test);
   });
+}
+template <class A>
+cudaError_t launch_plane_batch(int64_t n, const BatchZ& b, int count, int parseval, cudaStream_t st, int* nb) {
+  return dispatch_n(n, [&](auto t) { return Launch<A, decltype(t)::value>::plane_batch(b, count, parseval, st, nb); });
+}
+template <class A> cudaError_t launch_plane(const LaunchArgs& a, int* nb) {
+  return dispatch_n(a.n, [&](auto t) { return Launch<A, decltype(t)::value>::plane(a, nb); });
+}
+template <class A> bool has_plane(int64_t n) {
+  bool out = false;
+  dispatch_n(n, [&](auto t) {
+    out = Launch<A, decltype(t)::value>::has_plane();
+    return cudaSuccess;
+  });
+  return out;
 }
 template <class A> int launch_tma_xt(int64_t n) {
   int out = 0;

@@ -176,6 +176,39 @@ cudaError_t Launch<A, N>::zpass_batch(const BatchZ& b, int count, int parseval, 
 }
 
 template <class A, int N>
+bool Launch<A, N>::has_plane() {
+  return PlaneShape<A, N>::OK;
+}
+
+template <class A, int N>
+cudaError_t Launch<A, N>::plane_batch(const BatchZ& b, int count, int parseval, cudaStream_t st, int* nblocks) {
+  if constexpr (PlaneShape<A, N>::OK) {
+    using PS = PlaneShape<A, N>;
+    auto go = [&](auto kern) {
+      ensure_smem(kern, PS::SMEM);
+      pdl_launch(kern, dim3(N, count), PS::THREADS, PS::SMEM, st, b);
+    };
+    if (parseval) go(k_plane<A, N, true>);
+    else go(k_plane<A, N, false>);
+    if (nblocks) *nblocks = N;
+    return cudaGetLastError();
+  } else {
+    return cudaErrorInvalidValue;
+  }
+}
+
+template <class A, int N>
+cudaError_t Launch<A, N>::plane(const LaunchArgs& a, int* nblocks) {
+  BatchZ b{};
+  b.W[0] = a.W;
+  b.tw[0] = a.tw;
+  b.ktab[0] = a.ktab;
+  b.part[0] = a.part;
+  b.kp[0] = *a.kin;
+  return plane_batch(b, 1, a.stats, a.stream, nblocks);
+}
+
+template <class A, int N>
 cudaError_t Launch<A, N>::update_x_batch(const BatchU& b, int count, uint32_t scaled, int stats, int vx,
                                          cudaStream_t st, int* nblocks, int tma_test) {
   using C = typename A::C;
