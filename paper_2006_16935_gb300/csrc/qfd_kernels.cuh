@@ -498,18 +498,23 @@ __host__ __device__ constexpr int ilog2c(int n) { return n <= 1 ? 0 : 1 + ilog2c
 //   256, 32.16 for 512, 32.32 for 1024).  Four times the registers of R = 0
 //   for half the shared-memory exchanges: used by the complex64 y and z passes
 //   when the autotuner finds it faster.
+// Schedule R = 2 (N = 2^p with p >= 7, else as R = 0): E = 16; radix 16, 16, then
+//   N/256 (16.8 for 128): one exchange fewer than R = 0 and half its threads a
+//   line, for tiles twice as wide in the same CTA (complex64 pass A).
 template <int N, int R = 0> struct FftPlan {
   static constexpr bool R3 = N % 3 == 0;
   static constexpr int P2 = ilog2c(N);
   static constexpr bool TWO = R == 1 && !R3 && P2 >= 7;
-  static constexpr int E = TWO ? (1 << ((P2 + 1) / 2)) : (R3 ? 12 : 8);
+  static constexpr bool E16 = R == 2 && !R3 && P2 >= 7;
+  static constexpr int E = E16 ? 16 : TWO ? (1 << ((P2 + 1) / 2)) : (R3 ? 12 : 8);
   static constexpr int T = N / E;  // threads per line
   static constexpr int P = ilog2c(R3 ? N / 12 : N);
   static constexpr int Q = R3 ? P / 2 : P / 3;
   static constexpr int REM = R3 ? P % 2 : P % 3;
-  static constexpr int S = TWO ? 2 : (R3 ? 1 + Q + REM : Q + (REM ? 1 : 0));
+  static constexpr int S = E16 ? (P2 > 8 ? 3 : 2) : TWO ? 2 : (R3 ? 1 + Q + REM : Q + (REM ? 1 : 0));
   __host__ __device__ static constexpr int radix(int i) {
-    return TWO ? (i == 0 ? E : N / E) : R3 ? (i == 0 ? 12 : (i <= Q ? 4 : 2)) : (i < Q ? 8 : (REM == 1 ? 2 : 4));
+    return E16 ? (i == 0 ? 16 : i == 1 ? (N < 256 ? N / 16 : 16) : N / 256)
+           : TWO ? (i == 0 ? E : N / E) : R3 ? (i == 0 ? 12 : (i <= Q ? 4 : 2)) : (i < Q ? 8 : (REM == 1 ? 2 : 4));
   }
   __host__ __device__ static constexpr int ns(int i) { return i == 0 ? 1 : ns(i - 1) * radix(i - 1); }
 };
@@ -1061,9 +1066,16 @@ template <class A, int N> struct Shape {
   static constexpr bool WIDE = sizeof(typename A::C) >= 16;
   static constexpr int E = FftPlan<N>::E;  // elements per thread
   static constexpr int T = N / E;          // threads per line
-  static constexpr int XCOLS = TileCols<N, WIDE ? QFD_XCOLS_MIN16 : QFD_XCOLS_MIN8>::value;
+  // complex64 at 1024: 16 elements a thread (schedule 2) leave room for 16
+  // columns in a CTA.  Rows of 128 bytes instead of 64 at an 8 MB stride: pass A
+  // 13.65 -> 10.64 ms.  At 512, where a CTA holds 16 columns either way, schedule
+  // 2 is slower (0.92 -> 1.15 ms: psi and V must be loaded after the transform).
+  static constexpr int XR = A::id == 1 && N == 1024 ? 2 : 0;
+  static constexpr int XT = FftPlan<N, XR>::T;
+  static constexpr int XE = FftPlan<N, XR>::E;
+  static constexpr int XCOLS = XR == 2 ? 16 : TileCols<N, WIDE ? QFD_XCOLS_MIN16 : QFD_XCOLS_MIN8>::value;
   static constexpr int YCOLS = TileCols<N, WIDE ? QFD_YCOLS_MIN16 : QFD_YCOLS_MIN8>::value;
-  static constexpr int XTHREADS = T * XCOLS;
+  static constexpr int XTHREADS = XT * XCOLS;
   static constexpr int YTHREADS = T * YCOLS;
   static constexpr int XPITCH = XCOLS;  // shared-memory row pitch of the tiles
   static constexpr int YPITCH = YCOLS;
@@ -1481,29 +1493,30 @@ k_plane(const __grid_constant__ BatchZ b) {
 // column of W, psi and the update input already in registers, so that the
 // direct kernel (loads from global memory) and the TMA-staged one (loads from
 // shared memory) run the same arithmetic code.  XC is the tile width.
-template <class A, int N, int STATS, int XC>
-__device__ __forceinline__ void update_x_core(typename A::C (&v)[FftPlan<N>::E], const typename A::C (&ps)[FftPlan<N>::E],
-                                              const typename A::U (&cf)[FftPlan<N>::E], int t, int col, int64_t base,
+template <class A, int N, int STATS, int XC, int R>
+__device__ __forceinline__ void update_x_core(typename A::C (&v)[FftPlan<N, R>::E], const typename A::C (&ps)[FftPlan<N, R>::E],
+                                              const typename A::U (&cf)[FftPlan<N, R>::E], int t, int col, int64_t base,
                                               typename A::C* W, typename A::C* __restrict__ psi,
                                               const typename A::U* __restrict__ uin, const UpdParams& upar,
                                               const typename A::VT* __restrict__ V, const double* scale,
                                               const float* scale_f, const typename A::C* __restrict__ tw,
                                               typename A::C* sm, typename A::Acc& nacc, typename A::Full& facc) {
   using C = typename A::C;
-  using SH = Shape<A, N>;
+  using PL = FftPlan<N, R>;
   constexpr int64_t S = (int64_t)N * N;
-  using AT = AccTile<C, XC, SH::T>;
+  using AT = AccTile<C, XC, PL::T>;
   __shared__ int mxs[A::id == 0 ? AT::MAXN : 1];
   AT acc{sm, col, col, mxs};
-  fft_line<A, N, +1>(v, t, tw, acc);
+  fft_line<A, N, +1, AT, false, R>(v, t, tw, acc);
+  constexpr bool LATE = A::id == 0 || R == 2;
   const bool scaled = scale != nullptr;
   typename A::S s{};
   if (scaled) s = A::load_scale(scale, scale_f);
 #pragma unroll
-  for (int m = 0; m < SH::E; ++m) {
-    const int64_t idx = base + (t + m * SH::T) * S;
+  for (int m = 0; m < PL::E; ++m) {
+    const int64_t idx = base + (t + m * PL::T) * S;
     C nw;
-    if constexpr (A::id == 0) nw = A::update(psi[idx], v[m], A::coef_from(uin[idx], upar));
+    if constexpr (LATE) nw = A::update(psi[idx], v[m], A::coef_from(uin[idx], upar));
     else nw = A::update(ps[m], v[m], A::coef_from(cf[m], upar));
     if (scaled) nw = cscale(nw, s);
     psi[idx] = nw;
@@ -1511,14 +1524,14 @@ __device__ __forceinline__ void update_x_core(typename A::C (&v)[FftPlan<N>::E],
     if constexpr (STATS == STATS_NORM) nacc.add_norm(nw);
     if constexpr (STATS == STATS_FULL) facc.add(nw, V[idx]);
   }
-  fft_line<A, N, -1>(v, t, tw, acc);
+  fft_line<A, N, -1, AT, false, R>(v, t, tw, acc);
 #pragma unroll
-  for (int m = 0; m < SH::E; ++m) W[base + (t + m * SH::T) * S] = v[m];
+  for (int m = 0; m < PL::E; ++m) W[base + (t + m * PL::T) * S] = v[m];
 }
 
 // The direct pass A: psi and the per-site update input are loaded before the
 // inverse transform so that their latency overlaps it.
-template <class A, int N, int STATS, int XC>
+template <class A, int N, int STATS, int XC, int R>
 __device__ __forceinline__ void update_x_body(typename A::C* W, typename A::C* __restrict__ psi,
                                               const typename A::U* __restrict__ uin, const UpdParams& upar,
                                               const typename A::VT* __restrict__ V, const double* scale,
@@ -1526,39 +1539,39 @@ __device__ __forceinline__ void update_x_body(typename A::C* W, typename A::C* _
                                               double* __restrict__ part) {
   using C = typename A::C;
   using U = typename A::U;
-  using SH = Shape<A, N>;
+  using PL = FftPlan<N, R>;
   extern __shared__ __align__(16) unsigned char smraw[];
   C* sm = reinterpret_cast<C*>(smraw);
   const int col = threadIdx.x % XC, t = threadIdx.x / XC;
   const int64_t base = (int64_t)blockIdx.x * XC + col;
   constexpr int64_t S = (int64_t)N * N;
-  C v[SH::E], ps[SH::E];
-  U cf[SH::E];
+  C v[PL::E], ps[PL::E];
+  U cf[PL::E];
 #pragma unroll
-  for (int m = 0; m < SH::E; ++m) v[m] = W[base + (t + m * SH::T) * S];
-  if constexpr (A::id != 0) {  // (the fixed-point transforms leave no registers to hold them)
+  for (int m = 0; m < PL::E; ++m) v[m] = W[base + (t + m * PL::T) * S];
+  if constexpr (A::id != 0 && R != 2) {  // (else no registers are left to hold them)
 #pragma unroll
-    for (int m = 0; m < SH::E; ++m) ps[m] = psi[base + (t + m * SH::T) * S];
+    for (int m = 0; m < PL::E; ++m) ps[m] = psi[base + (t + m * PL::T) * S];
 #pragma unroll
-    for (int m = 0; m < SH::E; ++m) cf[m] = uin[base + (t + m * SH::T) * S];
+    for (int m = 0; m < PL::E; ++m) cf[m] = uin[base + (t + m * PL::T) * S];
   }
   typename A::Acc nacc;
   typename A::Full facc;
-  update_x_core<A, N, STATS, XC>(v, ps, cf, t, col, base, W, psi, uin, upar, V, scale, scale_f, tw, sm, nacc, facc);
+  update_x_core<A, N, STATS, XC, R>(v, ps, cf, t, col, base, W, psi, uin, upar, V, scale, scale_f, tw, sm, nacc, facc);
   if constexpr (STATS == STATS_NORM) norm_reduce_store<A>(nacc, part);
   if constexpr (STATS == STATS_FULL) full_store<A>(facc, part);
 }
 // Lattice i of the batch applies its pending normalisation factor when bit i
 // of `scaled` is set.  The half-width tiles (XC < XCOLS) are compiled for two
 // resident CTAs per SM.
-template <class A, int N, int STATS, int XC>
-__global__ void __launch_bounds__(N / FftPlan<N>::E * XC,
-                                  A::id == 0 ? ctas(N / FftPlan<N>::E * XC, 1024) : XC < Shape<A, N>::XCOLS ? 2 : 1)
+template <class A, int N, int STATS, int XC, int R = 0>
+__global__ void __launch_bounds__(FftPlan<N, R>::T * XC,
+                                  A::id == 0 || R == 2 ? ctas(FftPlan<N, R>::T * XC, 1024) : XC < Shape<A, N>::XCOLS ? ctas(FftPlan<N, R>::T * XC, 1024) : 1)
 k_update_x(const __grid_constant__ BatchU b, uint32_t scaled) {
   pdl_begin();
   using C = typename A::C;
   const int i = blockIdx.y;
-  update_x_body<A, N, STATS, XC>(static_cast<C*>(b.W[i]), static_cast<C*>(b.psi[i]),
+  update_x_body<A, N, STATS, XC, R>(static_cast<C*>(b.W[i]), static_cast<C*>(b.psi[i]),
                                  static_cast<const typename A::U*>(b.u[i]), b.up[i],
                                  static_cast<const typename A::VT*>(b.V[i]), (scaled >> i) & 1u ? b.scale[i] : nullptr,
                                  b.scale_f[i], static_cast<const C*>(b.tw[i]), b.part[i]);
@@ -1583,12 +1596,12 @@ k_forward_x(const typename A::C* src, typename A::C* W, typename A::C* psi_out, 
   const bool scaled = scale != nullptr;
   typename A::S s{};
   if (scaled) s = A::load_scale(scale, scale_f);
-  C v[SH::E];
+  C v[SH::XE];
   typename A::Acc nacc;
   typename A::Full facc;
 #pragma unroll
-  for (int m = 0; m < SH::E; ++m) {
-    const int64_t idx = base + (t + m * SH::T) * S;
+  for (int m = 0; m < SH::XE; ++m) {
+    const int64_t idx = base + (t + m * SH::XT) * S;
     C x = src[idx];
     if (scaled) x = cscale(x, s);
     v[m] = x;
@@ -1597,14 +1610,14 @@ k_forward_x(const typename A::C* src, typename A::C* W, typename A::C* psi_out, 
   }
   if (psi_out) {
 #pragma unroll
-    for (int m = 0; m < SH::E; ++m) psi_out[base + (t + m * SH::T) * S] = v[m];
+    for (int m = 0; m < SH::XE; ++m) psi_out[base + (t + m * SH::XT) * S] = v[m];
   }
-  using AT = AccTile<C, SH::XCOLS, SH::T>;
+  using AT = AccTile<C, SH::XCOLS, SH::XT>;
   __shared__ int mxs[A::id == 0 ? AT::MAXN : 1];
   AT acc{sm, col, col, mxs};
-  fft_line<A, N, -1>(v, t, tw, acc);
+  fft_line<A, N, -1, AT, false, SH::XR>(v, t, tw, acc);
 #pragma unroll
-  for (int m = 0; m < SH::E; ++m) W[base + (t + m * SH::T) * S] = v[m];
+  for (int m = 0; m < SH::XE; ++m) W[base + (t + m * SH::XT) * S] = v[m];
   if constexpr (STATS == STATS_NORM) norm_reduce_store<A>(nacc, part);
   if constexpr (STATS == STATS_FULL) full_store<A>(facc, part);
 }
@@ -1689,18 +1702,18 @@ k_project_x(const typename A::C* src, LowerPtrs lower, const double* sums, int k
       if (j < k) cc[j] = A::from_d2(double2{sums[2 * j], sums[2 * j + 1]});
   }
   // every load of the state and of its reflection is issued before any use
-  C v[SH::E], rv[SH::E];
+  C v[SH::XE], rv[SH::XE];
 #pragma unroll
-  for (int m = 0; m < SH::E; ++m) v[m] = src[base + (t + m * SH::T) * S];
+  for (int m = 0; m < SH::XE; ++m) v[m] = src[base + (t + m * SH::XT) * S];
   if (parity) {
 #pragma unroll
-    for (int m = 0; m < SH::E; ++m) rv[m] = src[rbase + (int64_t)reflect1<N>(t + m * SH::T, offgrid) * S];
+    for (int m = 0; m < SH::XE; ++m) rv[m] = src[rbase + (int64_t)reflect1<N>(t + m * SH::XT, offgrid) * S];
   }
   typename A::Acc nacc;
   typename A::Full facc;
 #pragma unroll
-  for (int m = 0; m < SH::E; ++m) {
-    const int x = t + m * SH::T;
+  for (int m = 0; m < SH::XE; ++m) {
+    const int x = t + m * SH::XT;
     const int64_t idx = base + x * S;
     C p = v[m];
     if (parity) p = A::half_comb(p, rv[m], parity);
@@ -1712,12 +1725,12 @@ k_project_x(const typename A::C* src, LowerPtrs lower, const double* sums, int k
     if constexpr (STATS == STATS_NORM) nacc.add_norm(p);
     if constexpr (STATS == STATS_FULL) facc.add(p, V[idx]);
   }
-  using AT = AccTile<C, SH::XCOLS, SH::T>;
+  using AT = AccTile<C, SH::XCOLS, SH::XT>;
   __shared__ int mxs[A::id == 0 ? AT::MAXN : 1];
   AT acc{sm, col, col, mxs};
-  fft_line<A, N, -1>(v, t, tw, acc);
+  fft_line<A, N, -1, AT, false, SH::XR>(v, t, tw, acc);
 #pragma unroll
-  for (int m = 0; m < SH::E; ++m) W[base + (t + m * SH::T) * S] = v[m];
+  for (int m = 0; m < SH::XE; ++m) W[base + (t + m * SH::XT) * S] = v[m];
   if constexpr (STATS == STATS_NORM) norm_reduce_store<A>(nacc, part);
   if constexpr (STATS == STATS_FULL) full_store<A>(facc, part);
 }

@@ -237,23 +237,23 @@ cudaError_t Launch<A, N>::update_x_batch(const BatchU& b, int count, uint32_t sc
       return cudaGetLastError();
     }
   }
-  auto go = [&](auto kern, int xc) {
+  auto go = [&](auto kern, int xc, int tpc) {
     const size_t smem = (size_t)N * xc * sizeof(C);
     const int grid = (int)((int64_t)N * N / xc);
     ensure_smem(kern, smem);
-    pdl_launch(kern, dim3(grid, count), SH::T * xc, smem, st, b, scaled);
+    pdl_launch(kern, dim3(grid, count), tpc * xc, smem, st, b, scaled);
     if (nblocks) *nblocks = grid;
   };
   if (vx == 1) {
     constexpr int XC = SH::XCOLS2;
-    if (stats == STATS_FULL) go(k_update_x<A, N, STATS_FULL, XC>, XC);
-    else if (stats == STATS_NORM) go(k_update_x<A, N, STATS_NORM, XC>, XC);
-    else go(k_update_x<A, N, STATS_NONE, XC>, XC);
+    if (stats == STATS_FULL) go(k_update_x<A, N, STATS_FULL, XC>, XC, SH::T);
+    else if (stats == STATS_NORM) go(k_update_x<A, N, STATS_NORM, XC>, XC, SH::T);
+    else go(k_update_x<A, N, STATS_NONE, XC>, XC, SH::T);
   } else {
-    constexpr int XC = SH::XCOLS;
-    if (stats == STATS_FULL) go(k_update_x<A, N, STATS_FULL, XC>, XC);
-    else if (stats == STATS_NORM) go(k_update_x<A, N, STATS_NORM, XC>, XC);
-    else go(k_update_x<A, N, STATS_NONE, XC>, XC);
+    constexpr int XC = SH::XCOLS, XR = SH::XR;
+    if (stats == STATS_FULL) go(k_update_x<A, N, STATS_FULL, XC, XR>, XC, SH::XT);
+    else if (stats == STATS_NORM) go(k_update_x<A, N, STATS_NORM, XC, XR>, XC, SH::XT);
+    else go(k_update_x<A, N, STATS_NONE, XC, XR>, XC, SH::XT);
   }
   return cudaGetLastError();
 }

@@ -171,7 +171,7 @@ k_update_x_tma(const __grid_constant__ BatchU b, uint32_t scaled, int test_skip)
     }
     __syncthreads();  // stage s is read: refill it with the tile after next
     if (tid == 0 && k + 2 * g < NT) issue(k + 2 * g, s);
-    update_x_core<A, N, STATS, XT>(v, ps, cf, t, col, (int64_t)k * XT + col, W, psi, nullptr, b.up[lat],
+    update_x_core<A, N, STATS, XT, 0>(v, ps, cf, t, col, (int64_t)k * XT + col, W, psi, nullptr, b.up[lat],
                                    static_cast<const typename A::VT*>(b.V[lat]), scale, b.scale_f[lat],
                                    static_cast<const C*>(b.tw[lat]), exch, nacc, facc);
   }
