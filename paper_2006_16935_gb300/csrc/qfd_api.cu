@@ -1535,6 +1535,9 @@ qfd_status qfd_plan(const qfd_params* params, qfd_plan_t* out) {
   pl->hist.assign(p.nstates, {});
   pl->arith16 = arith16_of(p.precision);
   pl->phase = uses32(p.precision) ? 1 : pl->arith16;
+  // complex64 y passes from n = 256 on start from the two-stage schedule (us, radix 8
+  // and two-stage: 256^3 53.8 and 46.3, 512^3 411 and 364, 1024^3 5150 and 3630)
+  if (n >= 256) pl->tune_vy[1] = 2;
 
   auto cleanup_fail = [&](qfd_status s, const std::string& msg) {
     g_create_error = msg;

@@ -31,6 +31,8 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <type_traits>
+
 namespace qfd {
 
 // ================================================== programmatic launches
@@ -839,6 +841,7 @@ __device__ __forceinline__ void stage_compute(typename A::C (&v)[FftPlan<N, R>::
 }
 
 // Writes stage outputs to their Stockham positions, then reads the canonical set.
+// Positions come as key(base) and a compile-time offset whose bits base has clear.
 template <typename C, int N, int R, int RAD, int NS, class Acc>
 __device__ __forceinline__ void stage_exchange(C (&v)[FftPlan<N, R>::E], int t, Acc& acc) {
   constexpr int E = FftPlan<N, R>::E;
@@ -846,13 +849,14 @@ __device__ __forceinline__ void stage_exchange(C (&v)[FftPlan<N, R>::E], int t, 
 #pragma unroll
   for (int u = 0; u < NB; ++u) {
     const int b = t + u * (N / E);
-    const int base = (b / NS) * NS * RAD + (b % NS);
+    const int base = acc.key((b / NS) * NS * RAD + (b % NS));
 #pragma unroll
-    for (int r = 0; r < RAD; ++r) acc.at(base + r * NS) = v[u + r * NB];
+    for (int r = 0; r < RAD; ++r) acc.at(base, r * NS) = v[u + r * NB];
   }
   acc.sync();
+  const int kt = acc.key(t);
 #pragma unroll
-  for (int m = 0; m < E; ++m) v[m] = acc.at(t + m * (N / E));
+  for (int m = 0; m < E; ++m) v[m] = acc.at(kt, m * (N / E));
   acc.sync();
 }
 
@@ -946,6 +950,8 @@ template <typename C, int CW, int T, int PITCH = CW> struct AccTile {
     return AccTile<D, CW, T, PITCH>(reinterpret_cast<D*>(sm), off, col);
   }
   __device__ __forceinline__ C& at(int pos) { return sm[pos * PITCH + off]; }
+  __device__ __forceinline__ int key(int base) const { return base; }
+  __device__ __forceinline__ C& at(int k, int c) { return at(k + c); }
   __device__ __forceinline__ void sync() { __syncthreads(); }
   __device__ __forceinline__ bool line_max(int& mx, bool odd, int t) {
 #pragma unroll
@@ -976,6 +982,8 @@ template <typename C, int PS, int T> struct AccLine {
     return AccLine<D, PS, T>(reinterpret_cast<D*>(sm), line);
   }
   __device__ __forceinline__ C& at(int pos) { return sm[pos + (pos >> PS)]; }
+  __device__ __forceinline__ int key(int base) const { return base; }
+  __device__ __forceinline__ C& at(int k, int c) { return at(k + c); }
   __device__ __forceinline__ void sync() {
     if constexpr (T <= 32) {
       __syncwarp();
@@ -999,6 +1007,27 @@ template <typename C, int PS, int T> struct AccLine {
 #pragma unroll
       for (int r = 0; r < WARPS; ++r) mx = max(mx, b[r]);
       return mx == 0x7fffffff;
+    }
+  }
+};
+
+// A line of complex64 in the z pass (N = 128..1024, radix-8 schedule): instead of
+// padding, bits 4, 5 and 6 of a position are folded into its four bank bits.
+// No padding serves both exchanges of this schedule (8-byte words: half a warp
+// per wavefront; the second exchange's writes took two), this fold does, for
+// one XOR an access (512^3 z pass 0.498 -> 0.475 ms).
+template <typename C, int T> struct AccLineX {
+  C* sm;
+  int line;
+  __device__ __forceinline__ AccLineX(C* s, int l) : sm(s), line(l) {}
+  static __device__ __forceinline__ constexpr int fold(int p) { return p ^ ((p >> 4) & 3) ^ (((p >> 6) & 1) * 12); }
+  __device__ __forceinline__ int key(int base) const { return fold(base); }
+  __device__ __forceinline__ C& at(int k, int c) { return sm[(k ^ (fold(c) & 15)) + (c & ~15)]; }
+  __device__ __forceinline__ void sync() {
+    if constexpr (T <= 32) {
+      __syncwarp();
+    } else {
+      asm volatile("bar.sync %0, %1;" ::"r"(1 + line), "r"(T) : "memory");
     }
   }
 };
@@ -1050,11 +1079,38 @@ __host__ __device__ constexpr int ctas(int threads, int resident) {
 }
 template <class A, int N, int ZG, int R> constexpr int z_resident() {
   if (A::id == 0) return ZG == 1 ? 1024 : 1;
-  if (A::id == 2) return ZG > 1 ? 1 : N % 3 == 0 ? 512 : N <= 64 ? 1024 : 768;
+  if (A::id == 2) return ZG > 1 ? 1 : N == 96 ? 512 : N <= 64 ? 1024 : 768;
   return R == 1 ? 384 : N % 3 == 0 || (ZG > 1 && N >= 512) ? 512 : ZG == 1 ? 768 : 640;
 }
 template <class A, int N, bool LOWER> constexpr int project_resident() {
   return A::id == 1 || (A::id == 0 && !LOWER) ? 1024 : A::id == 2 && !LOWER && N % 3 != 0 && N <= 256 ? 768 : 512;
+}
+// Pass A (us with and without the bound): complex64 1024 threads from n = 128 on
+// (256^3 137 -> 109, 128^3 16.7 -> 15.6; 64^3 is faster without, 7.2 against 8.2),
+// 768 at 96 and 192 (192^3 72 -> 47; 53 with 1024); double-float 512 (256^3 454 ->
+// 351, 128^3 56 -> 45, 96^3 34 -> 26; 377, 48 and 29 with 768), but 1024 from 512 on,
+// where two CTAs of 512 threads then fit (512^3 3.27 -> 2.97 ms).
+// x_late: psi and the update input are loaded where the update uses them instead
+// of before the inverse transform, so that their registers are free during it.
+template <class A, int N, int R> __host__ __device__ constexpr bool x_late() {
+  return A::id == 0 || R == 2 || (A::id == 2 && N >= 512);
+}
+template <class A, int N, int R> constexpr int x_resident() {
+  if (x_late<A, N, R>()) return 1024;
+  if (A::id == 2) return 512;
+  return N % 3 == 0 ? 768 : N >= 128 ? 1024 : 1;
+}
+// Complex64 y passes keep about 48 warps an SM (register-light transforms whose
+// exchanges need many warps in flight).  Double-float: 1024 threads from n = 256
+// on (512^3 1.25 -> 1.17 ms, 256^3 157 -> 140 us), 768 at 192 (78 -> 75), none
+// below (96^3 is slower with either).  The two-stage complex64 y pass: 512 threads
+// at 1024 (3.81 -> 3.63 ms), 768 at 256 (47.4 -> 46.3 us); at 512 any bound spills
+// (0.364 -> 0.384 ms with 512).
+template <class A, int N, int R> constexpr int y_resident() {
+  if (R == 1) return N == 1024 ? 512 : N == 256 ? 768 : 1;
+  if (A::id == 0) return 1024;
+  if (A::id == 1) return 1536;
+  return N % 3 == 0 ? (N >= 192 ? 768 : 1) : N >= 256 ? 1024 : 1;
 }
 template <int N, int CMIN> struct TileCols {
   static constexpr int T = N / FftPlan<N>::E;
@@ -1307,16 +1363,8 @@ __device__ __forceinline__ void fft_strided_body(typename A::C* W, const typenam
 #pragma unroll
   for (int m = 0; m < PL::E; ++m) W[base + (int64_t)(t + m * PL::T) * stride] = v[m];
 }
-// Resident CTAs per SM asked of the compiler for the y passes: complex64
-// keeps about 48 warps per SM (register-light transforms whose exchanges need
-// many warps in flight), the 16-byte arithmetics take what their registers allow.
-template <class A, int N, int YC> struct YOcc {
-  static constexpr int THREADS = N / FftPlan<N>::E * YC;
-  static constexpr int B0 = A::id == 1 ? 1536 / THREADS : A::id == 0 ? ctas(THREADS, 1024) : 1;
-  static constexpr int value = B0 < 1 ? 1 : (B0 > 8 ? 8 : B0);
-};
 template <class A, int N, int DIR, int YC, int R = 0>
-__global__ void __launch_bounds__(FftPlan<N, R>::T * YC, R == 0 ? YOcc<A, N, YC>::value : 1)
+__global__ void __launch_bounds__(FftPlan<N, R>::T * YC, ctas(FftPlan<N, R>::T * YC, y_resident<A, N, R>()))
 k_fft_strided(const __grid_constant__ BatchY b, int64_t stride, int tiles_inner, int64_t outer_stride) {
   using C = typename A::C;
   pdl_begin();
@@ -1331,6 +1379,12 @@ k_fft_strided(const __grid_constant__ BatchY b, int64_t stride, int tiles_inner,
 // next group are issued before the current group's transforms, so they are in
 // flight while it computes.
 // R: the radix schedule (FftPlan); LINES lines of T threads per CTA.
+template <class A, int N, int R> struct ZLine {
+  static constexpr bool FOLD = A::id == 1 && R == 0 && N >= 128 && N % 3 != 0;
+  using type = std::conditional_t<FOLD, AccLineX<typename A::C, FftPlan<N, R>::T>,
+                                  AccLine<typename A::C, R == 0 ? Shape<A, N>::PAD_SHIFT : Shape<A, N>::PAD_SHIFT_R1,
+                                          FftPlan<N, R>::T>>;
+};
 template <class A, int N, bool PARSEVAL, int ZG, int R, int LINES>
 __device__ __forceinline__ void zpass_body(typename A::C* W, const typename A::C* __restrict__ tw,
                                            const typename A::T* __restrict__ ktab, const KinParams& kp,
@@ -1349,9 +1403,12 @@ __device__ __forceinline__ void zpass_body(typename A::C* W, const typename A::C
   static_assert(PL::T <= 32 || LINES <= 15, "one named barrier per line");
   constexpr int PS = R == 0 ? SH::PAD_SHIFT : SH::PAD_SHIFT_R1;
   constexpr int LP = R == 0 ? SH::LPAD : SH::LPAD_R1;
-  using AL = AccLine<C, PS, PL::T>;
-  __shared__ int mxs[A::id == 0 ? AL::MAXN * LINES : 1];
-  AL acc{sm + l * LP, l, mxs};
+  using AL = typename ZLine<A, N, R>::type;
+  __shared__ int mxs[A::id == 0 ? AccLine<C, PS, PL::T>::MAXN * LINES : 1];
+  AL acc = [&] {
+    if constexpr (ZLine<A, N, R>::FOLD) return AL{sm + l * LP, l};
+    else return AL{sm + l * LP, l, mxs};
+  }();
   typename A::Pars pacc;
 #pragma unroll
   for (int g = 0; g < ZG; ++g) {
@@ -1508,7 +1565,6 @@ __device__ __forceinline__ void update_x_core(typename A::C (&v)[FftPlan<N, R>::
   __shared__ int mxs[A::id == 0 ? AT::MAXN : 1];
   AT acc{sm, col, col, mxs};
   fft_line<A, N, +1, AT, false, R>(v, t, tw, acc);
-  constexpr bool LATE = A::id == 0 || R == 2;
   const bool scaled = scale != nullptr;
   typename A::S s{};
   if (scaled) s = A::load_scale(scale, scale_f);
@@ -1516,7 +1572,7 @@ __device__ __forceinline__ void update_x_core(typename A::C (&v)[FftPlan<N, R>::
   for (int m = 0; m < PL::E; ++m) {
     const int64_t idx = base + (t + m * PL::T) * S;
     C nw;
-    if constexpr (LATE) nw = A::update(psi[idx], v[m], A::coef_from(uin[idx], upar));
+    if constexpr (x_late<A, N, R>()) nw = A::update(psi[idx], v[m], A::coef_from(uin[idx], upar));
     else nw = A::update(ps[m], v[m], A::coef_from(cf[m], upar));
     if (scaled) nw = cscale(nw, s);
     psi[idx] = nw;
@@ -1530,7 +1586,7 @@ __device__ __forceinline__ void update_x_core(typename A::C (&v)[FftPlan<N, R>::
 }
 
 // The direct pass A: psi and the per-site update input are loaded before the
-// inverse transform so that their latency overlaps it.
+// inverse transform so that their latency overlaps it (unless x_late).
 template <class A, int N, int STATS, int XC, int R>
 __device__ __forceinline__ void update_x_body(typename A::C* W, typename A::C* __restrict__ psi,
                                               const typename A::U* __restrict__ uin, const UpdParams& upar,
@@ -1549,7 +1605,7 @@ __device__ __forceinline__ void update_x_body(typename A::C* W, typename A::C* _
   U cf[PL::E];
 #pragma unroll
   for (int m = 0; m < PL::E; ++m) v[m] = W[base + (t + m * PL::T) * S];
-  if constexpr (A::id != 0 && R != 2) {  // (else no registers are left to hold them)
+  if constexpr (!x_late<A, N, R>()) {
 #pragma unroll
     for (int m = 0; m < PL::E; ++m) ps[m] = psi[base + (t + m * PL::T) * S];
 #pragma unroll
@@ -1562,11 +1618,10 @@ __device__ __forceinline__ void update_x_body(typename A::C* W, typename A::C* _
   if constexpr (STATS == STATS_FULL) full_store<A>(facc, part);
 }
 // Lattice i of the batch applies its pending normalisation factor when bit i
-// of `scaled` is set.  The half-width tiles (XC < XCOLS) are compiled for two
-// resident CTAs per SM.
+// of `scaled` is set. 
 template <class A, int N, int STATS, int XC, int R = 0>
 __global__ void __launch_bounds__(FftPlan<N, R>::T * XC,
-                                  A::id == 0 || R == 2 ? ctas(FftPlan<N, R>::T * XC, 1024) : XC < Shape<A, N>::XCOLS ? ctas(FftPlan<N, R>::T * XC, 1024) : 1)
+                                  ctas(FftPlan<N, R>::T * XC, x_resident<A, N, R>()))
 k_update_x(const __grid_constant__ BatchU b, uint32_t scaled) {
   pdl_begin();
   using C = typename A::C;
