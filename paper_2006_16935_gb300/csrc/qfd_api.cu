@@ -211,44 +211,85 @@ __device__ __forceinline__ int64_t lat_wrap(Lat L, int64_t c) {
 // all in FP64.  P-_{e_k} of Eq. (parity_axis), normalised as a projector:
 // (1/4) [psi(x) + psi(F_other x) - psi(F_k x) - psi(-x)], F_k the reflection of
 // axis k and F_other that of the two other axes.
+//
+// A thread takes the eight images of a site under the three axis reflections at
+// once: they share rho, sqrt and the volume test, every site is loaded once
+// instead of eight times, and the projections are sums over the eight sectors
+// u of the images' Walsh transform (sum over the images of |P psi|^2 is 1/8 the
+// sum of |u|^2 over the sectors P keeps: an even number of odd axes for P+, an
+// odd one for P-, {k odd} and {all odd} for P-_{e_k}).  The FP64 pipe bounds it:
+// about 75 operations a site become 9 to 16.  Coordinates that are their own
+// image (0 and n/2 with the on-grid centre) appear twice among the images, so
+// each orbit is weighted by its distinct sites / 8.
 template <class A>
 __global__ void __launch_bounds__(256)
 k_observables(const typename A::C* psi, Lat L, int offgrid, double half, double* __restrict__ part) {
   pdl_begin();
-  const int64_t n = L.n, n3 = n * n * n;
+  const int n = (int)L.n, h = offgrid ? n / 2 : n / 2 + 1;  // representatives 0..h-1 per axis
   const double cen = offgrid ? 0.5 * (double)(n - 1) : (double)(n / 2);
   double acc[NOBS];
 #pragma unroll
   for (int q = 0; q < NOBS; ++q) acc[q] = 0.0;
-  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n3; i += (int64_t)gridDim.x * blockDim.x) {
-    int64_t x, y, z;
-    lat_xyz(L, i, x, y, z);
-    const int64_t rx = offgrid ? n - 1 - x : lat_wrap(L, n - x), ry = offgrid ? n - 1 - y : lat_wrap(L, n - y),
-                  rz = offgrid ? n - 1 - z : lat_wrap(L, n - z);
-    const double2 p = A::to_d2(psi[i]), r = A::to_d2(psi[lat_idx(L, rx, ry, rz)]);
-    const double dx = (double)x - cen, dy = (double)y - cen, dz = (double)z - cen;
-    const double rho2 = dx * dx + dy * dy + dz * dz;
-    const double a2 = p.x * p.x + p.y * p.y;
-    acc[0] += a2;
-    acc[3] += rho2 * a2;
-    acc[4] += dx * a2;
-    acc[5] += dy * a2;
-    acc[6] += dz * a2;
-    if (fabs(dx) <= half && fabs(dy) <= half && fabs(dz) <= half) {
-      acc[1] += a2;
-      acc[2] += sqrt(rho2) * a2;
-      const double sx = 0.5 * (p.x + r.x), sy = 0.5 * (p.y + r.y), mx = 0.5 * (p.x - r.x), my = 0.5 * (p.y - r.y);
-      acc[7] += sx * sx + sy * sy;
-      acc[8] += mx * mx + my * my;
-      auto at = [&](int64_t X, int64_t Y, int64_t Z) { return A::to_d2(psi[lat_idx(L, X, Y, Z)]); };
-      const double2 f1 = at(rx, y, z), f2 = at(x, ry, z), f3 = at(x, y, rz);        // one axis reflected
-      const double2 g1 = at(x, ry, rz), g2 = at(rx, y, rz), g3 = at(rx, ry, z);     // the two others
-      const double2 fk[3] = {f1, f2, f3}, gk[3] = {g1, g2, g3};
+  const int total = h * h * h;
+  for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < total; i += gridDim.x * blockDim.x) {
+    const int c[3] = {i / (h * h), i / h % h, i % h};
+    int r[3];
+    bool two[3];  // the reflected coordinate is another one
+    double d[3];
 #pragma unroll
-      for (int k = 0; k < 3; ++k) {
-        const double ax = 0.25 * (p.x + gk[k].x - fk[k].x - r.x), ay = 0.25 * (p.y + gk[k].y - fk[k].y - r.y);
-        acc[9 + k] += ax * ax + ay * ay;
-      }
+    for (int k = 0; k < 3; ++k) {
+      r[k] = offgrid ? n - 1 - c[k] : (c[k] ? n - c[k] : 0);
+      two[k] = r[k] != c[k];
+      d[k] = (double)c[k] - cen;
+    }
+    double2 v[8];  // image abc (a, b, c = 1: reflected in x, y, z) at 4 a + 2 b + c
+    double a2[8];
+#pragma unroll
+    for (int m = 0; m < 8; ++m)
+      v[m] = A::to_d2(psi[lat_idx(L, m & 4 ? r[0] : c[0], m & 2 ? r[1] : c[1], m & 1 ? r[2] : c[2])]);
+#pragma unroll
+    for (int m = 0; m < 8; ++m) a2[m] = v[m].x * v[m].x + v[m].y * v[m].y;
+    const double w = (two[0] ? 1.0 : 0.5) * (two[1] ? 1.0 : 0.5) * (two[2] ? 1.0 : 0.5);
+    // sums and differences of |psi|^2 along z, y, x
+    double s1[4], s2[2], dz = 0.0, dy = 0.0;
+#pragma unroll
+    for (int m = 0; m < 4; ++m) {
+      s1[m] = a2[2 * m] + a2[2 * m + 1];
+      dz += a2[2 * m] - a2[2 * m + 1];
+    }
+#pragma unroll
+    for (int m = 0; m < 2; ++m) {
+      s2[m] = s1[2 * m] + s1[2 * m + 1];
+      dy += s1[2 * m] - s1[2 * m + 1];
+    }
+    const double all = s2[0] + s2[1], dx = s2[0] - s2[1], wa = w * all;
+    const double rho2 = d[0] * d[0] + d[1] * d[1] + d[2] * d[2];
+    acc[0] += wa;
+    acc[3] += rho2 * wa;
+    acc[4] += d[0] * (w * (two[0] ? dx : all));
+    acc[5] += d[1] * (w * (two[1] ? dy : all));
+    acc[6] += d[2] * (w * (two[2] ? dz : all));
+    if (fabs(d[0]) <= half && fabs(d[1]) <= half && fabs(d[2]) <= half) {
+      acc[1] += wa;
+      acc[2] += sqrt(rho2) * wa;
+#pragma unroll
+      for (int o = 1; o < 8; o <<= 1)
+#pragma unroll
+        for (int m = 0; m < 8; ++m)
+          if (!(m & o)) {
+            const double2 p = v[m], q = v[m | o];
+            v[m] = double2{p.x + q.x, p.y + q.y};
+            v[m | o] = double2{p.x - q.x, p.y - q.y};
+          }
+      double u[8];
+#pragma unroll
+      for (int m = 0; m < 8; ++m) u[m] = v[m].x * v[m].x + v[m].y * v[m].y;
+      const double w8 = 0.125 * w;
+      acc[7] += w8 * ((u[0] + u[3]) + (u[5] + u[6]));
+      acc[8] += w8 * ((u[1] + u[2]) + (u[4] + u[7]));
+      acc[9] += w8 * (u[4] + u[7]);
+      acc[10] += w8 * (u[2] + u[7]);
+      acc[11] += w8 * (u[1] + u[7]);
     }
   }
   block_reduce_store<NOBS>(acc, part);
