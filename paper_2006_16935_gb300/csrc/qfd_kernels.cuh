@@ -1694,35 +1694,55 @@ __device__ __forceinline__ int reflect1(int x, int offgrid) {
 
 // Overlaps <phi_j | P psi> for j < k (P the parity projector of Eq. (parity),
 // the identity for parity 0), summed per CTA in the policy's exact
-// accumulator and stored as FP64 partials (2 per lower state).
-template <class A, int N>
+// accumulator and stored as FP64 partials (2 per lower state).  K >= k is the
+// compiled number of accumulators; each thread takes U sites a turn, all of
+// whose loads are issued before the first sum (the sums are long dependent
+// chains: with one site a turn and eight accumulators the loads were exposed;
+// 256^3 with two lower states: complex64 225 -> 125 us, complex128 1.71 -> 0.58 ms).
+template <class A, int N, int K>
 __global__ void __launch_bounds__(256)
 k_gs_dots(const typename A::C* psi, LowerPtrs lower, int k, int parity, int offgrid,
           double* __restrict__ part) {
   pdl_begin();
   using C = typename A::C;
   constexpr int64_t N3 = (int64_t)N * N * N;
-  typename A::Dot acc[MAX_LOWER];
-  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < N3; i += (int64_t)gridDim.x * blockDim.x) {
-    C p = psi[i];
-    if (parity) {
-      const int z = (int)(i % N), y = (int)((i / N) % N), x = (int)(i / ((int64_t)N * N));
-      const int64_t ri = ((int64_t)reflect1<N>(x, offgrid) * N + reflect1<N>(y, offgrid)) * N +
-                         reflect1<N>(z, offgrid);
-      p = A::half_comb(p, psi[ri], parity);
+  constexpr int U = (sizeof(C) == 8 ? 8 : 4) / K > 4 ? 4 : (sizeof(C) == 8 ? 8 : 4) / K > 1 ? (sizeof(C) == 8 ? 8 : 4) / K : 1;
+  typename A::Dot acc[K];
+  const int64_t step = (int64_t)gridDim.x * blockDim.x;
+  for (int64_t i0 = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i0 < N3; i0 += U * step) {
+    C p[U], q[U], f[K][U];
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+      const int64_t i = i0 + u * step;
+      if (i < N3) {
+        p[u] = psi[i];
+        if (parity) {
+          const int z = (int)(i % N), y = (int)((i / N) % N), x = (int)(i / ((int64_t)N * N));
+          q[u] = psi[((int64_t)reflect1<N>(x, offgrid) * N + reflect1<N>(y, offgrid)) * N + reflect1<N>(z, offgrid)];
+        }
+#pragma unroll
+        for (int j = 0; j < K; ++j)
+          if (j < k) f[j][u] = static_cast<const C*>(lower.p[j])[i];
+      }
     }
 #pragma unroll
-    for (int j = 0; j < MAX_LOWER; ++j)
-      if (j < k) acc[j].add(static_cast<const C*>(lower.p[j])[i], p);
-  }
-  double q[2 * MAX_LOWER];
+    for (int u = 0; u < U; ++u) {
+      if (i0 + u * step < N3) {
+        const C x = parity ? A::half_comb(p[u], q[u], parity) : p[u];
 #pragma unroll
-  for (int j = 0; j < MAX_LOWER; ++j) {
+        for (int j = 0; j < K; ++j)
+          if (j < k) acc[j].add(f[j][u], x);
+      }
+    }
+  }
+  double q[2 * K];
+#pragma unroll
+  for (int j = 0; j < K; ++j) {
     const double2 d = acc[j].value();
     q[2 * j] = d.x;
     q[2 * j + 1] = d.y;
   }
-  block_reduce_store<2 * MAX_LOWER>(q, part);
+  block_reduce_store<2 * K>(q, part);
 }
 
 // The cadence's projection fused with the forward x transform: psi' = P psi -

@@ -105,8 +105,12 @@ template <class A, int N>
 cudaError_t Launch<A, N>::gs_dots(const LaunchArgs& a, int nblocks) {
   LowerPtrs lp;
   for (int j = 0; j < MAX_LOWER; ++j) lp.p[j] = a.lower[j];
-  return pdl_launch(k_gs_dots<A, N>, nblocks, 256, 0, a.stream, (const typename A::C*)a.src, lp, a.k, a.parity,
-                    a.offgrid, a.part);
+  auto go = [&](auto kern) {
+    return pdl_launch(kern, nblocks, 256, 0, a.stream, (const typename A::C*)a.src, lp, a.k, a.parity, a.offgrid,
+                      a.part);
+  };
+  return a.k <= 1 ? go(k_gs_dots<A, N, 1>) : a.k <= 2 ? go(k_gs_dots<A, N, 2>)
+         : a.k <= 4 ? go(k_gs_dots<A, N, 4>) : go(k_gs_dots<A, N, MAX_LOWER>);
 }
 
 template <class A, int N>
