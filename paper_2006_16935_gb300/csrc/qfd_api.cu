@@ -303,6 +303,23 @@ __global__ void k_convert(const typename AI::C* in, typename AO::C* out, int64_t
 }
 
 // ------------------------------------------------ finite-difference H_K(0)
+// The sum of six doubles with one rounding, on integers: every term is aligned to
+// the largest exponent of the six (2^-59 of it is kept; FP64 additions round five
+// times at 2^-53).  The FP64 pipe bounds the complex128 stencil, and its ten
+// additions a site are most of what it does.  Terms outside the exponents covered
+// (non-finite, huge, all tiny or zero) are added in FP64.
+__device__ __forceinline__ double sum6(const double (&v)[6]) {
+  int E = 0;
+#pragma unroll
+  for (int j = 0; j < 6; ++j) E = max(E, __double2hiint(v[j]) & 0x7fffffff);
+  E >>= 20;
+  if (E < FX_E_MIN || E > FX_E_MAX) return v[0] + v[1] + v[2] + v[3] + v[4] + v[5];
+  long long s = 0;
+#pragma unroll
+  for (int j = 0; j < 6; ++j) s += fx_in<6>(v[j], E);
+  return fx_out(s, E - 1081);
+}
+
 // H_K(0) psi at site idx of the n^3 lattice with psi = 0 outside it
 // (Eq. HK0 with Dirichlet boundaries, normalised as its momentum-space form,
 // Eq. HK0_momentum_space_1): c (6 psi - the sum of the six neighbours) with
@@ -316,13 +333,25 @@ __device__ __forceinline__ typename A::C fdtd_sum(const typename A::C* psi, int6
   lat_xyz(L, idx, x, y, z);
   const C zero{};
   self = psi[idx];
-  C s = x > 0 ? psi[idx - n2] : zero;
-  s = cadd(s, x + 1 < n ? psi[idx + n2] : zero);
-  s = cadd(s, y > 0 ? psi[idx - n] : zero);
-  s = cadd(s, y + 1 < n ? psi[idx + n] : zero);
-  s = cadd(s, z > 0 ? psi[idx - 1] : zero);
-  s = cadd(s, z + 1 < n ? psi[idx + 1] : zero);
-  return s;
+  if constexpr (A::id == 1) {  // one term at a time: registers for more threads (512^3 0.64 ms, 0.92 with all six loaded)
+    C s = x > 0 ? psi[idx - n2] : zero;
+    s = cadd(s, x + 1 < n ? psi[idx + n2] : zero);
+    s = cadd(s, y > 0 ? psi[idx - n] : zero);
+    s = cadd(s, y + 1 < n ? psi[idx + n] : zero);
+    s = cadd(s, z > 0 ? psi[idx - 1] : zero);
+    return cadd(s, z + 1 < n ? psi[idx + 1] : zero);
+  }
+  const C q[6] = {x > 0 ? psi[idx - n2] : zero, x + 1 < n ? psi[idx + n2] : zero, y > 0 ? psi[idx - n] : zero,
+                  y + 1 < n ? psi[idx + n] : zero, z > 0 ? psi[idx - 1] : zero, z + 1 < n ? psi[idx + 1] : zero};
+  if constexpr (A::id == 0) {
+    return C{sum6({q[0].x, q[1].x, q[2].x, q[3].x, q[4].x, q[5].x}),
+             sum6({q[0].y, q[1].y, q[2].y, q[3].y, q[4].y, q[5].y})};
+  } else {
+    C s = q[0];
+#pragma unroll
+    for (int j = 1; j < 6; ++j) s = cadd(s, q[j]);
+    return s;
+  }
 }
 template <class A>
 __device__ __forceinline__ typename A::C fdtd_hk(const typename A::C* psi, int64_t idx, Lat L,
@@ -349,9 +378,10 @@ k_fdtd_update(const typename A::C* psi, typename A::C* __restrict__ out,
   if (scaled) s = A::load_scale(scale, scale_f);
   typename A::Acc nacc;
   typename A::Full facc;
-  // sites per thread unrolled in the stencil loop (measured at 512^3: four
-  // for the 16-byte arithmetics, one for complex64)
-  constexpr int U = A::id == 1 ? 1 : 4;
+  // sites per thread unrolled in the stencil loop (measured at 512^3: four for
+  // double-float, one for complex64, six for complex128: 256^3 440 us with two,
+  // 364 with four, 340 with six, 345 with eight, and 516 with FP64 sums)
+  constexpr int U = A::id == 1 ? 1 : A::id == 0 ? 6 : 4;
 #pragma unroll U
   for (int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; idx < n3; idx += (int64_t)gridDim.x * blockDim.x) {
     C self;
@@ -374,6 +404,8 @@ k_fdtd_energy(const typename A::C* psi, Lat L, typename A::S c, double* __restri
   using C = typename A::C;
   const int64_t n3 = L.n * L.n * L.n;
   double e = 0.0;
+  constexpr int U = A::id == 0 ? 4 : 1;  // (complex128 256^3: 606 us without, 390 with four)
+#pragma unroll U
   for (int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; idx < n3; idx += (int64_t)gridDim.x * blockDim.x) {
     C self;
     const C hk = fdtd_hk<A>(psi, idx, L, c, self);

@@ -96,3 +96,39 @@ def test_every_shape_gives_the_same_bits(qfdlib, n):
     outs = [step(n, psi, V, 2, t) for t in [(0, -1, 0), (1, 0, 0), (0, 1, 1)]]
     for o in outs[1:]:
         assert rel(o, outs[0]) < 1e-15
+
+
+def fdtd_reference(n, psi, V, dt):
+    s = np.zeros_like(psi)
+    for ax in range(3):
+        lo = [slice(None)] * 3
+        hi = [slice(None)] * 3
+        lo[ax], hi[ax] = slice(0, n - 1), slice(1, n)
+        s[tuple(hi)] += psi[tuple(lo)]
+        s[tuple(lo)] += psi[tuple(hi)]
+    h = 0.5 * dt * V
+    return (1 - h) / (1 + h) * psi - dt / (1 + h) * (6 * psi - s) / (2 * M * A * A)
+
+
+@pytest.mark.parametrize("n", [8, 96, 128])
+@pytest.mark.parametrize("kind", ["noise", "delta", "decay", "planes"])
+def test_stencil_sums_match_site_by_site(qfdlib, n, kind):
+    # the neighbour sum on integers: within a few rounding errors of its largest
+    # term at every site (also where the six span many scales, or are all zero)
+    V = O.potential(n, A, "cornell", (0.3, 0.2), "offgrid")
+    psi = states(n, kind)
+    dt = 0.5 * 2 * M * A * A / 12
+    with Q.Plan(n, A, M, dt, 0, ortho_every=1000, centre="offgrid") as p:
+        p.set_potential(V)
+        p.set_psi(0, psi)
+        p.step(0, 1)
+        got = p.get_psi(0)
+    want = fdtd_reference(n, psi, V, dt)
+    big = np.abs(psi)
+    pad = np.pad(big, 1)
+    for ax in range(3):
+        for sh in (0, 2):
+            w = [slice(1, n + 1)] * 3
+            w[ax] = slice(sh, sh + n)
+            big = np.maximum(big, pad[tuple(w)])
+    assert np.all(np.abs(got - want) <= 16 * 2.0 ** -53 * big + 1e-300)
