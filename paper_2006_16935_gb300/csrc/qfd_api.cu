@@ -127,6 +127,16 @@ __global__ void k_potential(double* __restrict__ V, int64_t n, double a, int kin
   }
 }
 
+// T(k)/N^3 (FP64) for kx, ky, kz < h = N/2 + 1, in the order and with the
+// operations of the z pass.
+__global__ void k_kin_octant(const double* __restrict__ ktab, KinParams kp, int h, double* __restrict__ out) {
+  const int64_t h3 = (int64_t)h * h * h;
+  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < h3; i += (int64_t)gridDim.x * blockDim.x) {
+    const int z = (int)(i % h), y = (int)(i / h % h), x = (int)(i / ((int64_t)h * h));
+    out[i] = F64::kin(F64::kadd(F64::kadd(ktab[x], ktab[y]), ktab[z]), kp);
+  }
+}
+
 // Update coefficients of Sec. 2.2 from V, per arithmetic: FP64 {A, B dtau}
 // (complex128 pass A reads them precomputed); for H_K(0) plans also FP32 and
 // double-float {B dtau, 1 - A} with 1 - A = dtau V B formed in FP64 (the FFT
@@ -496,6 +506,7 @@ struct qfd_plan_s {
   float2* tw32 = nullptr;
   dfc* twdf = nullptr;
   double* ktab64 = nullptr;
+  double* ttab64 = nullptr;  // T(k)/N^3 of an octant (complex128 plans of the FFT terms)
   float* ktab32 = nullptr;
   df* ktabdf = nullptr;
   double* partA = nullptr;
@@ -675,6 +686,7 @@ LaunchArgs base_args(qfd_plan_t pl) {
   a.W = pl->W;
   a.tw = tw_of<A>(pl);
   a.ktab = ktab_of<A>(pl);
+  a.ttab = A::id == 0 ? pl->ttab64 : nullptr;
   a.kin = &pl->kin;
   a.coef = uin_of<A>(pl);
   a.up = &pl->up;
@@ -1284,6 +1296,11 @@ int arith16_of(int precision) { return (precision == QFD_DF64 || precision == QF
 // pass A, and every 16-byte H_K(0) update), the complex64 H_K(0) coefficients,
 // and V in FP32 (complex64 pass A of the FFT terms).
 bool needs_coef16(const qfd_params& p) { return uses16(p.precision) && (arith16_of(p.precision) == 0 || p.kinetic == 0); }
+// T(k)/N^3 of the octant kx, ky, kz <= n/2 (the complex128 z pass)
+size_t ttab_bytes(const qfd_params& p) {
+  const size_t h = (size_t)p.n / 2 + 1;
+  return uses16(p.precision) && arith16_of(p.precision) == 0 && p.kinetic != 0 ? h * h * h * sizeof(double) : 0;
+}
 bool needs_coef32(const qfd_params& p) { return uses32(p.precision) && p.kinetic == 0; }
 bool needs_v32(const qfd_params& p) { return uses32(p.precision) && p.kinetic != 0; }
 // Device bytes a plan with these parameters allocates (lattices, tables, partials).
@@ -1298,7 +1315,7 @@ size_t plan_device_bytes(const qfd_params& p) {
   if (needs_coef32(p)) b += n3 * 8;
   if (needs_v32(p)) b += n3 * sizeof(float);
   if (uses_vdf(p.precision)) b += n3 * sizeof(df);
-  return b;
+  return b + ttab_bytes(p);
 }
 bool uses32(int precision) {
   return precision == QFD_C64 || precision == QFD_C64_REFINE || precision == QFD_C64_REFINE_DF;
@@ -1334,6 +1351,7 @@ qfd_status batch_step_once(qfd_plan_s* const* pls, const int* ss, int count, int
       by.W[nx] = bz.W[nx] = pl->W;
       by.tw[nx] = bz.tw[nx] = tw_of<A>(pl);
       bz.ktab[nx] = ktab_of<A>(pl);
+      bz.ttab[nx] = A::id == 0 ? pl->ttab64 : nullptr;
       bz.kp[nx] = pl->kin;
       ++nx;
     } else if ((r = advance_to_d<A>(pl, 0)) != QFD_OK) {
@@ -1444,6 +1462,7 @@ qfd_status batch_period_launch(qfd_plan_s* const* pls, const int* ss, int count,
     by.W[i] = bz.W[i] = pl->W;
     by.tw[i] = bz.tw[i] = tw_of<A>(pl);
     bz.ktab[i] = ktab_of<A>(pl);
+    bz.ttab[i] = A::id == 0 ? pl->ttab64 : nullptr;
     bz.kp[i] = pl->kin;
     bz.part[i] = pl->partC;
   }
@@ -1650,6 +1669,7 @@ qfd_status qfd_plan(const qfd_params* params, qfd_plan_t* out) {
   };
   if (uses16(p.precision)) allocs.push_back({(void**)&pl->psi16, (size_t)(p.nstates + 1) * n3 * 16});
   if (uses32(p.precision)) allocs.push_back({(void**)&pl->psi32, (size_t)(p.nstates + 1) * n3 * sizeof(float2)});
+  if (ttab_bytes(p)) allocs.push_back({(void**)&pl->ttab64, ttab_bytes(p)});
   if (needs_coef16(p)) allocs.push_back({(void**)&pl->coef16, (size_t)n3 * 16});
   if (needs_coef32(p)) allocs.push_back({(void**)&pl->coef32, (size_t)n3 * sizeof(float2)});
   if (needs_v32(p)) allocs.push_back({(void**)&pl->V32, (size_t)n3 * sizeof(float)});
@@ -1691,6 +1711,11 @@ qfd_status qfd_plan(const qfd_params* params, qfd_plan_t* out) {
             cudaMemcpy(pl->ktab32, kt32.data(), n * sizeof(float), cudaMemcpyHostToDevice) == cudaSuccess &&
             cudaMemcpy(pl->ktabdf, ktdf.data(), n * sizeof(df), cudaMemcpyHostToDevice) == cudaSuccess &&
             cudaMemset(pl->scal, 0, SC_COUNT * sizeof(double)) == cudaSuccess;
+  if (ok && pl->ttab64) {
+    const int h = (int)n / 2 + 1;
+    k_kin_octant<<<grid_for((int64_t)h * h * h), 256, 0, pl->st>>>(pl->ktab64, pl->kin, h, pl->ttab64);
+    ok = cudaGetLastError() == cudaSuccess && cudaStreamSynchronize(pl->st) == cudaSuccess;
+  }
   if (!ok) return cleanup_fail(QFD_ERR_CUDA, "table upload failed");
   if (cudaHostAlloc((void**)&pl->hscal, (SC_COUNT + 1) * sizeof(double), cudaHostAllocDefault) != cudaSuccess)
     return cleanup_fail(QFD_ERR_OOM, "pinned host buffer allocation failed");
@@ -1707,7 +1732,7 @@ void qfd_destroy(qfd_plan_t pl) {
   if (!pl) return;
   if (pl->st) cudaStreamSynchronize(pl->st);
   void* bufs[] = {pl->psi16, pl->psi32, pl->W,      pl->coef16, pl->coef32, pl->V,     pl->tw64,
-                  pl->tw32,  pl->twdf,  pl->ktab64, pl->ktab32, pl->ktabdf, pl->partA, pl->partC,
+                  pl->tw32,  pl->twdf,  pl->ktab64, pl->ttab64, pl->ktab32, pl->ktabdf, pl->partA, pl->partC,
                   pl->partG, pl->scal,  pl->scalf, pl->flag, pl->Vdf, pl->V32, pl->errflag, pl->tmaps};
   for (void* b : bufs)
     if (b) cudaFree(b);

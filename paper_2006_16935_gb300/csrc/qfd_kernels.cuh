@@ -1315,6 +1315,7 @@ struct BatchZ {  // pass C
   const void* ktab[MAX_BATCH];
   double* part[MAX_BATCH];  // Parseval partials (energy checks)
   KinParams kp[MAX_BATCH];
+  const void* ttab[MAX_BATCH];  // complex128: T(k)/N^3 of an octant (kin_octant), or null
 };
 struct BatchU {  // pass A
   void* W[MAX_BATCH];
@@ -1379,6 +1380,28 @@ k_fft_strided(const __grid_constant__ BatchY b, int64_t stride, int tiles_inner,
 // next group are issued before the current group's transforms, so they are in
 // flight while it computes.
 // R: the radix schedule (FftPlan); LINES lines of T threads per CTA.
+// T(k)/N^3 of one z line (kx, ky).  T is even along every axis, so complex128
+// plans hold it for the octant kx, ky, kz <= N/2 (N/2 + 1 entries an axis, 1/16 of
+// a lattice of complex128) and read it instead of spending 2 (HK1, HK2) or about 12
+// (HK3) operations a site on the FP64 pipe, which bounds this pass.  512^3 z pass:
+// HK2 2.58 -> 2.50 ms; HK3, which took 1.7 times as long as HK2, takes the same 2.50.
+// The values are those that kin gives.
+template <int N> __device__ __forceinline__ int kin_octant(int j) { return j <= N / 2 ? j : N - j; }
+template <class A, int N> struct KinLine {
+  using T = typename A::T;
+  const T* ktab;
+  const T* row;
+  T sxy;
+  __device__ __forceinline__ KinLine(const T* kt, const T* ttab, int kx, int ky) : ktab(kt), row(nullptr) {
+    constexpr int H = N / 2 + 1;
+    if (A::id == 0 && ttab) row = ttab + ((int64_t)kin_octant<N>(kx) * H + kin_octant<N>(ky)) * H;
+    else sxy = A::kadd(ktab[kx], ktab[ky]);
+  }
+  __device__ __forceinline__ T at(int kz, const KinParams& kp) const {
+    if (A::id == 0 && row) return row[kin_octant<N>(kz)];
+    return A::kin(A::kadd(sxy, ktab[kz]), kp);
+  }
+};
 template <class A, int N, int R> struct ZLine {
   static constexpr bool FOLD = A::id == 1 && R == 0 && N >= 128 && N % 3 != 0;
   using type = std::conditional_t<FOLD, AccLineX<typename A::C, FftPlan<N, R>::T>,
@@ -1387,7 +1410,8 @@ template <class A, int N, int R> struct ZLine {
 };
 template <class A, int N, bool PARSEVAL, int ZG, int R, int LINES>
 __device__ __forceinline__ void zpass_body(typename A::C* W, const typename A::C* __restrict__ tw,
-                                           const typename A::T* __restrict__ ktab, const KinParams& kp,
+                                           const typename A::T* __restrict__ ktab,
+                                           const typename A::T* __restrict__ ttab, const KinParams& kp,
                                            double* __restrict__ part) {
   using C = typename A::C;
   using T = typename A::T;
@@ -1420,10 +1444,10 @@ __device__ __forceinline__ void zpass_body(typename A::C* W, const typename A::C
       for (int m = 0; m < PL::E; ++m) nx[m] = p[(int64_t)LINES * N + t + m * PL::T];
     }
     fft_line<A, N, -1, decltype(acc), true, R>(v, t, tw, acc);
-    const T sxy = A::kadd(ktab[line / N], ktab[line % N]);
+    const KinLine<A, N> kin(ktab, ttab, (int)(line / N), (int)(line % N));
 #pragma unroll
     for (int m = 0; m < PL::E; ++m) {
-      const T tk = A::kin(A::kadd(sxy, ktab[t + m * PL::T]), kp);
+      const T tk = kin.at(t + m * PL::T, kp);
       if constexpr (PARSEVAL) pacc.add(tk, v[m]);
       v[m] = cscale(v[m], tk);
     }
@@ -1448,7 +1472,8 @@ k_zpass(const __grid_constant__ BatchZ b) {
   using C = typename A::C;
   const int i = blockIdx.y;
   zpass_body<A, N, PARSEVAL, ZG, R, ZLines<A, N, R>::value>(static_cast<C*>(b.W[i]), static_cast<const C*>(b.tw[i]),
-                                                             static_cast<const typename A::T*>(b.ktab[i]), b.kp[i],
+                                                             static_cast<const typename A::T*>(b.ktab[i]),
+                                                             static_cast<const typename A::T*>(b.ttab[i]), b.kp[i],
                                                              b.part[i]);
 }
 
@@ -1516,10 +1541,10 @@ k_plane(const __grid_constant__ BatchZ b) {
     for (int m = 0; m < E; ++m) v[m] = acc.at(tz + m * TT);
     acc.sync();
     fft_line<A, N, -1, AL, true>(v, tz, tw, acc);
-    const T sxy = A::kadd(ktab[x], ktab[l]);
+    const KinLine<A, N> kin(ktab, static_cast<const T*>(b.ttab[lat]), x, l);
 #pragma unroll
     for (int m = 0; m < E; ++m) {
-      const T tk = A::kin(A::kadd(sxy, ktab[tz + m * TT]), kp);
+      const T tk = kin.at(tz + m * TT, kp);
       if constexpr (PARSEVAL) pacc.add(tk, v[m]);
       v[m] = cscale(v[m], tk);
     }

@@ -71,6 +71,7 @@ cudaError_t Launch<A, N>::zpass(const LaunchArgs& a, int* nblocks) {
   b.W[0] = a.W;
   b.tw[0] = a.tw;
   b.ktab[0] = a.ktab;
+  b.ttab[0] = a.ttab;
   b.part[0] = a.part;
   b.kp[0] = *a.kin;
   return zpass_batch(b, 1, a.stats, a.vz, a.stream, nblocks);
@@ -207,6 +208,7 @@ cudaError_t Launch<A, N>::plane(const LaunchArgs& a, int* nblocks) {
   b.W[0] = a.W;
   b.tw[0] = a.tw;
   b.ktab[0] = a.ktab;
+  b.ttab[0] = a.ttab;
   b.part[0] = a.part;
   b.kp[0] = *a.kin;
   return plane_batch(b, 1, a.stats, a.stream, nblocks);
