@@ -45,10 +45,8 @@ constexpr int FIN_THREADS = 1024;
 namespace qfd {
 
 // Fixed-order sums of per-CTA partials, then the derived scalars of `op`.
-__global__ void __launch_bounds__(FIN_THREADS)
-k_finalize_op(const double* part, int nq, int count, double* scal, float* scalf,
-              int op) {
-  pdl_begin();
+__device__ __forceinline__ void finalize_body(const double* part, int nq, int count, double* scal, float* scalf,
+                                              int op) {
   __shared__ double red[32];
   __shared__ double sums[2 * MAX_LOWER];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -127,13 +125,47 @@ __global__ void k_potential(double* __restrict__ V, int64_t n, double a, int kin
   }
 }
 
-// T(k)/N^3 (FP64) for kx, ky, kz < h = N/2 + 1, in the order and with the
-// operations of the z pass.
-__global__ void k_kin_octant(const double* __restrict__ ktab, KinParams kp, int h, double* __restrict__ out) {
+__global__ void __launch_bounds__(FIN_THREADS)
+k_finalize_op(const double* part, int nq, int count, double* scal, float* scalf, int op) {
+  pdl_begin();
+  finalize_body(part, nq, count, scal, scalf, op);
+}
+
+// The same for the lattices of a batch, one CTA each (a launch per lattice took
+// about 2 us of the batch's stream), and their normalisation factors applied.
+struct BatchF {
+  const double* part[MAX_BATCH];
+  double* scal[MAX_BATCH];
+  float* scalf[MAX_BATCH];
+};
+__global__ void __launch_bounds__(FIN_THREADS)
+k_finalize_batch(const __grid_constant__ BatchF b, int nq, int count, int op) {
+  pdl_begin();
+  const int i = blockIdx.x;
+  finalize_body(b.part[i], nq, count, b.scal[i], b.scalf[i], op);
+}
+struct BatchS {
+  void* psi[MAX_BATCH];
+  const double* scale[MAX_BATCH];
+};
+template <class A> __global__ void k_scale_batch(const __grid_constant__ BatchS b, int64_t n3) {
+  pdl_begin();
+  const int l = blockIdx.y;
+  typename A::C* psi = static_cast<typename A::C*>(b.psi[l]);
+  const typename A::S fs = A::scalar(b.scale[l][0]);
+  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n3; i += (int64_t)gridDim.x * blockDim.x)
+    psi[i] = cscale(psi[i], fs);
+}
+
+// T(k)/N^3 for kx, ky, kz < h = N/2 + 1, in the order and with the operations of
+// the z pass.
+template <class A>
+__global__ void k_kin_octant(const typename A::T* __restrict__ ktab, KinParams kp, int h,
+                             typename A::T* __restrict__ out) {
   const int64_t h3 = (int64_t)h * h * h;
   for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < h3; i += (int64_t)gridDim.x * blockDim.x) {
     const int z = (int)(i % h), y = (int)(i / h % h), x = (int)(i / ((int64_t)h * h));
-    out[i] = F64::kin(F64::kadd(F64::kadd(ktab[x], ktab[y]), ktab[z]), kp);
+    out[i] = A::kin(A::kadd(A::kadd(ktab[x], ktab[y]), ktab[z]), kp);
   }
 }
 
@@ -506,7 +538,7 @@ struct qfd_plan_s {
   float2* tw32 = nullptr;
   dfc* twdf = nullptr;
   double* ktab64 = nullptr;
-  double* ttab64 = nullptr;  // T(k)/N^3 of an octant (complex128 plans of the FFT terms)
+  void* ttab = nullptr;      // T(k)/N^3 of an octant, FP64 or double-float (16-byte plans of the FFT terms)
   float* ktab32 = nullptr;
   df* ktabdf = nullptr;
   double* partA = nullptr;
@@ -686,7 +718,7 @@ LaunchArgs base_args(qfd_plan_t pl) {
   a.W = pl->W;
   a.tw = tw_of<A>(pl);
   a.ktab = ktab_of<A>(pl);
-  a.ttab = A::id == 0 ? pl->ttab64 : nullptr;
+  a.ttab = A::id == 0 ? pl->ttab : nullptr;
   a.kin = &pl->kin;
   a.coef = uin_of<A>(pl);
   a.up = &pl->up;
@@ -730,6 +762,20 @@ const void* psi_tmap(qfd_plan_t pl, const void* p) {
 qfd_status finalize(qfd_plan_t pl, const double* part, int nq, int count, int op) {
   QFD_RUN(PASS_FINALIZE,
           pdl_launch(k_finalize_op, 1, FIN_THREADS, 0, pl->st, part, nq, count, pl->scal, pl->scalf, op));
+  return QFD_OK;
+}
+
+// finalize for several plans' partials of pass A (or C) in one launch on p0's stream.
+qfd_status finalize_batch(qfd_plan_t p0, const std::vector<qfd_plan_t>& pls, bool pass_c, int nq, int count, int op) {
+  if (pls.empty()) return QFD_OK;
+  BatchF b{};
+  for (size_t i = 0; i < pls.size(); ++i) {
+    b.part[i] = pass_c ? pls[i]->partC : pls[i]->partA;
+    b.scal[i] = pls[i]->scal;
+    b.scalf[i] = pls[i]->scalf;
+  }
+  qfd_plan_t pl = p0;
+  QFD_RUN(PASS_FINALIZE, pdl_launch(k_finalize_batch, (int)pls.size(), FIN_THREADS, 0, pl->st, b, nq, count, op));
   return QFD_OK;
 }
 
@@ -1296,7 +1342,7 @@ int arith16_of(int precision) { return (precision == QFD_DF64 || precision == QF
 // pass A, and every 16-byte H_K(0) update), the complex64 H_K(0) coefficients,
 // and V in FP32 (complex64 pass A of the FFT terms).
 bool needs_coef16(const qfd_params& p) { return uses16(p.precision) && (arith16_of(p.precision) == 0 || p.kinetic == 0); }
-// T(k)/N^3 of the octant kx, ky, kz <= n/2 (the complex128 z pass)
+// T(k)/N^3 of the octant kx, ky, kz <= n/2 (the 16-byte z pass)
 size_t ttab_bytes(const qfd_params& p) {
   const size_t h = (size_t)p.n / 2 + 1;
   return uses16(p.precision) && arith16_of(p.precision) == 0 && p.kinetic != 0 ? h * h * h * sizeof(double) : 0;
@@ -1351,7 +1397,7 @@ qfd_status batch_step_once(qfd_plan_s* const* pls, const int* ss, int count, int
       by.W[nx] = bz.W[nx] = pl->W;
       by.tw[nx] = bz.tw[nx] = tw_of<A>(pl);
       bz.ktab[nx] = ktab_of<A>(pl);
-      bz.ttab[nx] = A::id == 0 ? pl->ttab64 : nullptr;
+      bz.ttab[nx] = A::id == 0 ? pl->ttab : nullptr;
       bz.kp[nx] = pl->kin;
       ++nx;
     } else if ((r = advance_to_d<A>(pl, 0)) != QFD_OK) {
@@ -1415,16 +1461,27 @@ qfd_status batch_step_once(qfd_plan_s* const* pls, const int* ss, int count, int
     pl->pending = false;
     pl->t[ss[i]] += 1;
   }
+  // the scalars of the lattices that only normalise, or only take an energy
+  // check, in one launch each; the others' cadences one by one
+  std::vector<qfd_plan_t> norm, n2pv;
+  for (int i = 0; i < count; ++i) {
+    qfd_plan_t pl = pls[i];
+    if (pl->t[ss[i]] % pl->p.ortho_every == 0) {
+      if (!projects(pl, ss[i])) norm.push_back(pl);
+    } else if (check) {
+      n2pv.push_back(pl);
+    }
+  }
+  if ((r = finalize_batch(p0, norm, false, 2, nb, OP_NORM)) != QFD_OK) return r;
+  for (qfd_plan_t pl : norm) pl->pending = true;
+  if ((r = finalize_batch(p0, n2pv, false, 2, nb, OP_N2PV)) != QFD_OK) return r;
   for (int i = 0; i < count; ++i) {
     qfd_plan_t pl = pls[i];
     const int s = ss[i];
-    if (pl->t[s] % pl->p.ortho_every == 0) {
-      if ((r = cadence<A>(pl, s, check)) != QFD_OK) return r;
-      if (pl->snap_every > 0 && s == 0 && pl->t[s] % pl->snap_every == 0 && (r = take_snapshot<A>(pl)) != QFD_OK)
-        return r;
-    } else if (check) {
-      if ((r = finalize(pl, pl->partA, 2, pl->nA, OP_N2PV)) != QFD_OK) return r;
-    }
+    if (pl->t[s] % pl->p.ortho_every != 0) continue;
+    if (projects(pl, s) && (r = cadence<A>(pl, s, check)) != QFD_OK) return r;
+    if (pl->snap_every > 0 && s == 0 && pl->t[s] % pl->snap_every == 0 && (r = take_snapshot<A>(pl)) != QFD_OK)
+      return r;
   }
   return QFD_OK;
 }
@@ -1435,8 +1492,26 @@ qfd_status step_batch(qfd_plan_s* const* pls, const int* ss, int count, int64_t 
   qfd_status r;
   for (int64_t it = 0; it < nsteps; ++it)
     if ((r = batch_step_once<A>(pls, ss, count, 0, pls[0]->st)) != QFD_OK) return r;
-  for (int i = 0; i < count; ++i)
-    if ((r = materialize<A>(pls[i], ss[i])) != QFD_OK) return r;
+  // the pending normalisations (materialize) in one launch
+  BatchS b{};
+  int ns = 0;
+  for (int i = 0; i < count; ++i) {
+    qfd_plan_t pl = pls[i];
+    if (!pl->pending) continue;
+    b.psi[ns] = psi_of<A>(pl, ss[i]);
+    b.scale[ns++] = pl->scal + SC_SCALE;
+  }
+  if (ns > 0) {
+    qfd_plan_t pl = pls[0];
+    const int64_t n3 = pl->n3;
+    const int g = std::max(1, (grid_for(n3) + ns - 1) / ns);
+    QFD_RUN(PASS_OTHER, pdl_launch(k_scale_batch<A>, dim3(g, ns), 256, 0, pl->st, b, n3));
+    for (int i = 0; i < count; ++i)
+      if (pls[i]->pending) {
+        pls[i]->pending = false;
+        pls[i]->w_stage = ST_NONE;
+      }
+  }
   return QFD_OK;
 }
 
@@ -1462,7 +1537,7 @@ qfd_status batch_period_launch(qfd_plan_s* const* pls, const int* ss, int count,
     by.W[i] = bz.W[i] = pl->W;
     by.tw[i] = bz.tw[i] = tw_of<A>(pl);
     bz.ktab[i] = ktab_of<A>(pl);
-    bz.ttab[i] = A::id == 0 ? pl->ttab64 : nullptr;
+    bz.ttab[i] = A::id == 0 ? pl->ttab : nullptr;
     bz.kp[i] = pl->kin;
     bz.part[i] = pl->partC;
   }
@@ -1481,7 +1556,10 @@ qfd_status batch_period_launch(qfd_plan_s* const* pls, const int* ss, int count,
     qfd_plan_t pl = pls[i];
     pl->nC = nc;
     pl->w_stage = plane_path<A>(p0) ? ST_D : ST_C;
-    if ((r = finalize(pl, pl->partC, 1, pl->nC, OP_ENERGY)) != QFD_OK) return r;
+  }
+  if ((r = finalize_batch(p0, std::vector<qfd_plan_t>(pls, pls + count), true, 1, nc, OP_ENERGY)) != QFD_OK) return r;
+  for (int i = 0; i < count; ++i) {
+    qfd_plan_t pl = pls[i];
     QFD_CK(cudaMemcpyAsync(pl->hscal, pl->scal, SC_COUNT * sizeof(double), cudaMemcpyDeviceToHost, st));
     QFD_CK(cudaMemcpyAsync(pl->hscal + SC_COUNT, pl->errflag, sizeof(int), cudaMemcpyDeviceToHost, st));
   }
@@ -1669,7 +1747,7 @@ qfd_status qfd_plan(const qfd_params* params, qfd_plan_t* out) {
   };
   if (uses16(p.precision)) allocs.push_back({(void**)&pl->psi16, (size_t)(p.nstates + 1) * n3 * 16});
   if (uses32(p.precision)) allocs.push_back({(void**)&pl->psi32, (size_t)(p.nstates + 1) * n3 * sizeof(float2)});
-  if (ttab_bytes(p)) allocs.push_back({(void**)&pl->ttab64, ttab_bytes(p)});
+  if (ttab_bytes(p)) allocs.push_back({(void**)&pl->ttab, ttab_bytes(p)});
   if (needs_coef16(p)) allocs.push_back({(void**)&pl->coef16, (size_t)n3 * 16});
   if (needs_coef32(p)) allocs.push_back({(void**)&pl->coef32, (size_t)n3 * sizeof(float2)});
   if (needs_v32(p)) allocs.push_back({(void**)&pl->V32, (size_t)n3 * sizeof(float)});
@@ -1711,9 +1789,11 @@ qfd_status qfd_plan(const qfd_params* params, qfd_plan_t* out) {
             cudaMemcpy(pl->ktab32, kt32.data(), n * sizeof(float), cudaMemcpyHostToDevice) == cudaSuccess &&
             cudaMemcpy(pl->ktabdf, ktdf.data(), n * sizeof(df), cudaMemcpyHostToDevice) == cudaSuccess &&
             cudaMemset(pl->scal, 0, SC_COUNT * sizeof(double)) == cudaSuccess;
-  if (ok && pl->ttab64) {
+  if (ok && pl->ttab) {
     const int h = (int)n / 2 + 1;
-    k_kin_octant<<<grid_for((int64_t)h * h * h), 256, 0, pl->st>>>(pl->ktab64, pl->kin, h, pl->ttab64);
+    const int g = grid_for((int64_t)h * h * h);
+    if (pl->arith16 == 0) k_kin_octant<F64><<<g, 256, 0, pl->st>>>(pl->ktab64, pl->kin, h, (double*)pl->ttab);
+    else k_kin_octant<DF><<<g, 256, 0, pl->st>>>(pl->ktabdf, pl->kin, h, (df*)pl->ttab);
     ok = cudaGetLastError() == cudaSuccess && cudaStreamSynchronize(pl->st) == cudaSuccess;
   }
   if (!ok) return cleanup_fail(QFD_ERR_CUDA, "table upload failed");
@@ -1732,7 +1812,7 @@ void qfd_destroy(qfd_plan_t pl) {
   if (!pl) return;
   if (pl->st) cudaStreamSynchronize(pl->st);
   void* bufs[] = {pl->psi16, pl->psi32, pl->W,      pl->coef16, pl->coef32, pl->V,     pl->tw64,
-                  pl->tw32,  pl->twdf,  pl->ktab64, pl->ttab64, pl->ktab32, pl->ktabdf, pl->partA, pl->partC,
+                  pl->tw32,  pl->twdf,  pl->ktab64, pl->ttab, pl->ktab32, pl->ktabdf, pl->partA, pl->partC,
                   pl->partG, pl->scal,  pl->scalf, pl->flag, pl->Vdf, pl->V32, pl->errflag, pl->tmaps};
   for (void* b : bufs)
     if (b) cudaFree(b);
