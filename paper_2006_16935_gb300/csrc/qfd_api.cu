@@ -718,7 +718,7 @@ LaunchArgs base_args(qfd_plan_t pl) {
   a.W = pl->W;
   a.tw = tw_of<A>(pl);
   a.ktab = ktab_of<A>(pl);
-  a.ttab = A::id == 0 ? pl->ttab : nullptr;
+  a.ttab = A::id != 1 ? pl->ttab : nullptr;
   a.kin = &pl->kin;
   a.coef = uin_of<A>(pl);
   a.up = &pl->up;
@@ -1345,7 +1345,7 @@ bool needs_coef16(const qfd_params& p) { return uses16(p.precision) && (arith16_
 // T(k)/N^3 of the octant kx, ky, kz <= n/2 (the 16-byte z pass)
 size_t ttab_bytes(const qfd_params& p) {
   const size_t h = (size_t)p.n / 2 + 1;
-  return uses16(p.precision) && arith16_of(p.precision) == 0 && p.kinetic != 0 ? h * h * h * sizeof(double) : 0;
+  return uses16(p.precision) && p.kinetic != 0 ? h * h * h * sizeof(double) : 0;
 }
 bool needs_coef32(const qfd_params& p) { return uses32(p.precision) && p.kinetic == 0; }
 bool needs_v32(const qfd_params& p) { return uses32(p.precision) && p.kinetic != 0; }
@@ -1397,7 +1397,7 @@ qfd_status batch_step_once(qfd_plan_s* const* pls, const int* ss, int count, int
       by.W[nx] = bz.W[nx] = pl->W;
       by.tw[nx] = bz.tw[nx] = tw_of<A>(pl);
       bz.ktab[nx] = ktab_of<A>(pl);
-      bz.ttab[nx] = A::id == 0 ? pl->ttab : nullptr;
+      bz.ttab[nx] = A::id != 1 ? pl->ttab : nullptr;
       bz.kp[nx] = pl->kin;
       ++nx;
     } else if ((r = advance_to_d<A>(pl, 0)) != QFD_OK) {
@@ -1537,7 +1537,7 @@ qfd_status batch_period_launch(qfd_plan_s* const* pls, const int* ss, int count,
     by.W[i] = bz.W[i] = pl->W;
     by.tw[i] = bz.tw[i] = tw_of<A>(pl);
     bz.ktab[i] = ktab_of<A>(pl);
-    bz.ttab[i] = A::id == 0 ? pl->ttab : nullptr;
+    bz.ttab[i] = A::id != 1 ? pl->ttab : nullptr;
     bz.kp[i] = pl->kin;
     bz.part[i] = pl->partC;
   }

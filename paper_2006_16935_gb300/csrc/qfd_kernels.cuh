@@ -1112,9 +1112,9 @@ template <class A, int N, int R> constexpr int y_resident() {
   if (A::id == 1) return 1536;
   return N % 3 == 0 ? (N >= 192 ? 768 : 1) : N >= 256 ? 1024 : 1;
 }
-template <int N, int CMIN> struct TileCols {
+template <int N, int CMIN, int TARGET = QFD_TILE_TARGET> struct TileCols {
   static constexpr int T = N / FftPlan<N>::E;
-  static constexpr int C0 = (QFD_TILE_TARGET / T > CMIN) ? QFD_TILE_TARGET / T : CMIN;
+  static constexpr int C0 = (TARGET / T > CMIN) ? TARGET / T : CMIN;
   static constexpr int C1 = C0 < 1024 / T ? C0 : 1024 / T;
   static constexpr int value = C1 < N ? C1 : N;
 };
@@ -1129,8 +1129,9 @@ template <class A, int N> struct Shape {
   static constexpr int XR = A::id == 1 && N == 1024 ? 2 : 0;
   static constexpr int XT = FftPlan<N, XR>::T;
   static constexpr int XE = FftPlan<N, XR>::E;
-  static constexpr int XCOLS = XR == 2 ? 16 : TileCols<N, WIDE ? QFD_XCOLS_MIN16 : QFD_XCOLS_MIN8>::value;
-  static constexpr int YCOLS = TileCols<N, WIDE ? QFD_YCOLS_MIN16 : QFD_YCOLS_MIN8>::value;
+  static constexpr int TT = QFD_TILE_TARGET;
+  static constexpr int XCOLS = XR == 2 ? 16 : TileCols<N, WIDE ? QFD_XCOLS_MIN16 : QFD_XCOLS_MIN8, TT>::value;
+  static constexpr int YCOLS = TileCols<N, WIDE ? QFD_YCOLS_MIN16 : QFD_YCOLS_MIN8, TT>::value;
   static constexpr int XTHREADS = XT * XCOLS;
   static constexpr int YTHREADS = T * YCOLS;
   static constexpr int XPITCH = XCOLS;  // shared-memory row pitch of the tiles
@@ -1315,7 +1316,7 @@ struct BatchZ {  // pass C
   const void* ktab[MAX_BATCH];
   double* part[MAX_BATCH];  // Parseval partials (energy checks)
   KinParams kp[MAX_BATCH];
-  const void* ttab[MAX_BATCH];  // complex128: T(k)/N^3 of an octant (kin_octant), or null
+  const void* ttab[MAX_BATCH];  // 16-byte sites: T(k)/N^3 of an octant (kin_octant), or null
 };
 struct BatchU {  // pass A
   void* W[MAX_BATCH];
@@ -1385,7 +1386,8 @@ k_fft_strided(const __grid_constant__ BatchY b, int64_t stride, int tiles_inner,
 // a lattice of complex128) and read it instead of spending 2 (HK1, HK2) or about 12
 // (HK3) operations a site on the FP64 pipe, which bounds this pass.  512^3 z pass:
 // HK2 2.58 -> 2.50 ms; HK3, which took 1.7 times as long as HK2, takes the same 2.50.
-// The values are those that kin gives.
+// The values are those that kin gives.  Double-float plans hold it too (512^3 z pass
+// 2.63 -> 2.56 ms with HK2, 2.76 -> 2.56 with HK3).
 template <int N> __device__ __forceinline__ int kin_octant(int j) { return j <= N / 2 ? j : N - j; }
 template <class A, int N> struct KinLine {
   using T = typename A::T;
@@ -1394,11 +1396,11 @@ template <class A, int N> struct KinLine {
   T sxy;
   __device__ __forceinline__ KinLine(const T* kt, const T* ttab, int kx, int ky) : ktab(kt), row(nullptr) {
     constexpr int H = N / 2 + 1;
-    if (A::id == 0 && ttab) row = ttab + ((int64_t)kin_octant<N>(kx) * H + kin_octant<N>(ky)) * H;
+    if (A::id != 1 && ttab) row = ttab + ((int64_t)kin_octant<N>(kx) * H + kin_octant<N>(ky)) * H;
     else sxy = A::kadd(ktab[kx], ktab[ky]);
   }
   __device__ __forceinline__ T at(int kz, const KinParams& kp) const {
-    if (A::id == 0 && row) return row[kin_octant<N>(kz)];
+    if (A::id != 1 && row) return row[kin_octant<N>(kz)];
     return A::kin(A::kadd(sxy, ktab[kz]), kp);
   }
 };

@@ -113,7 +113,7 @@ struct LaunchArgs {
   const float* scale_f = nullptr;  // its FP32 rounding and double-float split
   const void* tw = nullptr;    // twiddles exp(-2 pi i e / N), e < N
   const void* ktab = nullptr;  // per-axis kinetic table
-  const void* ttab = nullptr;  // T(k)/N^3 of an octant (complex128) or null
+  const void* ttab = nullptr;  // T(k)/N^3 of an octant (16-byte sites) or null
   const KinParams* kin = nullptr;
   double* part = nullptr;      // per-CTA partials
   int stats = 0;               // STATS_* for passes A / forward x, Parseval flag for pass C
