@@ -1112,6 +1112,9 @@ template <class A, int N, int R> constexpr int y_resident() {
   if (A::id == 1) return 1536;
   return N % 3 == 0 ? (N >= 192 ? 768 : 1) : N >= 256 ? 1024 : 1;
 }
+// TARGET threads a tile: 64 instead of 256 for complex128 up to n = 96, so that
+// small lattices spread over all SMs (us a step: 64^3 29.9 -> 29.0, 96^3 75.5 -> 69.4;
+// 128^3 is slower, 130.0 -> 131.2).
 template <int N, int CMIN, int TARGET = QFD_TILE_TARGET> struct TileCols {
   static constexpr int T = N / FftPlan<N>::E;
   static constexpr int C0 = (TARGET / T > CMIN) ? TARGET / T : CMIN;
@@ -1129,7 +1132,7 @@ template <class A, int N> struct Shape {
   static constexpr int XR = A::id == 1 && N == 1024 ? 2 : 0;
   static constexpr int XT = FftPlan<N, XR>::T;
   static constexpr int XE = FftPlan<N, XR>::E;
-  static constexpr int TT = QFD_TILE_TARGET;
+  static constexpr int TT = A::id == 0 && N <= 96 ? 64 : QFD_TILE_TARGET;
   static constexpr int XCOLS = XR == 2 ? 16 : TileCols<N, WIDE ? QFD_XCOLS_MIN16 : QFD_XCOLS_MIN8, TT>::value;
   static constexpr int YCOLS = TileCols<N, WIDE ? QFD_YCOLS_MIN16 : QFD_YCOLS_MIN8, TT>::value;
   static constexpr int XTHREADS = XT * XCOLS;
