@@ -940,6 +940,7 @@ template <typename C, int CW, int T, int PITCH = CW> struct AccTile {
   static constexpr int G = CW >= 32 ? 1 : (32 / CW < T ? 32 / CW : T);  // threads of a column in a warp
   static constexpr int ROWS = T / G;                                       // partial maxima of a column
   static constexpr int MAXN = 2 * ROWS * CW;
+  static constexpr unsigned LANES = CW * T >= 32 ? 0xffffffffu : (1u << (CW * T % 32)) - 1;  // (tiles of under 32 threads)
   C* sm;
   int off, col;
   int* mxs;
@@ -955,7 +956,7 @@ template <typename C, int CW, int T, int PITCH = CW> struct AccTile {
   __device__ __forceinline__ void sync() { __syncthreads(); }
   __device__ __forceinline__ bool line_max(int& mx, bool odd, int t) {
 #pragma unroll
-    for (int o = CW; o < CW * G; o <<= 1) mx = max(mx, __shfl_xor_sync(0xffffffffu, mx, o));
+    for (int o = CW; o < CW * G; o <<= 1) mx = max(mx, __shfl_xor_sync(LANES, mx, o));
     int* b = mxs + flip;
     flip = flip ? 0 : ROWS * CW;
     if (t % G == 0) b[t / G * CW + col] = mx;
@@ -996,7 +997,7 @@ template <typename C, int PS, int T> struct AccLine {
     if constexpr (T <= 32) {
 #pragma unroll
       for (int o = 1; o < T; o <<= 1) mx = max(mx, __shfl_xor_sync(0xffffffffu, mx, o));
-      return __any_sync(__activemask(), odd);
+      return __any_sync(__activemask(), odd);  // (a block of n = 8 planes has eight lanes)
     } else {
       if (odd) mx = 0x7fffffff;
       mx = __reduce_max_sync(0xffffffffu, mx);
