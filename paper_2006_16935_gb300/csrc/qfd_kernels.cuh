@@ -4,6 +4,9 @@
 // (Eqs. HK1-HK3) is four passes over the N^3 lattice (layout [x][y][z], z
 // contiguous, interleaved complex):
 //
+// (where a plane x = const fits in shared memory, B, C and D are one launch:
+// k_plane)
+//
 //   pass A  x-lines : inverse DFT_x of W  -> H_K psi, the A/B update of Sec. 2.2,
 //                     norm / <V> partial sums, forward DFT_x of the new psi -> W
 //   pass B  y-lines : forward DFT_y of W (in place)
@@ -217,7 +220,7 @@ struct F64 {
   // the normalisation factor as written by the reduction kernel: FP64 value,
   // then its FP32 rounding and double-float split in a float array
   static __device__ __forceinline__ S load_scale(const double* d, const float*) { return *d; }
-  // complex128 passes are bound by FP64 issue, so the coefficients are read
+  // the complex128 pass A is short of FP64 issue, so the coefficients are read
   // precomputed (16 B) rather than derived per site with an FP64 division
   static __device__ __forceinline__ K coef_from(U u, const UpdParams&) { return u; }
   // Eq. (iter_proced) as printed: A psi - (B dtau) H_K psi
@@ -703,8 +706,9 @@ template <int RAD, int DIR, typename C> __device__ __forceinline__ void dft_smal
   if constexpr (RAD == 8) dft8<DIR>(x);
 }
 
-// Twiddled radix-8 butterfly of the complex128 stages with scaled twiddles
-// (the tangent form of Linzer and Feig).  Each twiddle is w_r = s_r q_r with
+// Twiddled radix-8 butterfly of the FP64 transform (the complex128 lines that
+// fixed point does not cover) with scaled twiddles (the tangent form of Linzer
+// and Feig).  Each twiddle is w_r = s_r q_r with
 // q_r = 1 + i tan(theta_r) where |cos| >= |sin|, else q_r = cot(theta_r) + i,
 // so |s_r| >= 1/sqrt 2 and |tan|, |cot| <= 1.  x_r q_r takes two FMAs, and the
 // real factors s_r enter, as ratios, the multiply-adds that replace the
@@ -1136,6 +1140,12 @@ template <class A, int N> struct Shape {
   static constexpr int TT = A::id == 0 && N <= 96 ? 64 : QFD_TILE_TARGET;
   static constexpr int XCOLS = XR == 2 ? 16 : TileCols<N, WIDE ? QFD_XCOLS_MIN16 : QFD_XCOLS_MIN8, TT>::value;
   static constexpr int YCOLS = TileCols<N, WIDE ? QFD_YCOLS_MIN16 : QFD_YCOLS_MIN8, TT>::value;
+  // forward x alone holds nothing but the line: schedule 2 from 512 on (two CTAs of
+  // 512 threads an SM; 512^3 complex64 0.767 -> 0.623 ms, no gain at 256)
+  static constexpr int FR = A::id == 1 && N >= 512 ? 2 : 0;
+  static constexpr int FT = FftPlan<N, FR>::T;
+  static constexpr int FE = FftPlan<N, FR>::E;
+  static constexpr int FTHREADS = FT * XCOLS;
   static constexpr int XTHREADS = XT * XCOLS;
   static constexpr int YTHREADS = T * YCOLS;
   static constexpr int XPITCH = XCOLS;  // shared-memory row pitch of the tiles
@@ -1667,7 +1677,7 @@ k_update_x(const __grid_constant__ BatchU b, uint32_t scaled) {
 // psi_out) into W; partials per STATS of the scaled input.  src may alias W
 // (each CTA reads its whole tile before writing it).
 template <class A, int N, int STATS>
-__global__ void __launch_bounds__(Shape<A, N>::XTHREADS, ctas(Shape<A, N>::XTHREADS, 1024))
+__global__ void __launch_bounds__(Shape<A, N>::FTHREADS, ctas(Shape<A, N>::FTHREADS, 1024))
 k_forward_x(const typename A::C* src, typename A::C* W, typename A::C* psi_out, const typename A::VT* __restrict__ V,
             const double* scale, const float* scale_f, const typename A::C* __restrict__ tw,
             double* __restrict__ part) {
@@ -1682,12 +1692,12 @@ k_forward_x(const typename A::C* src, typename A::C* W, typename A::C* psi_out, 
   const bool scaled = scale != nullptr;
   typename A::S s{};
   if (scaled) s = A::load_scale(scale, scale_f);
-  C v[SH::XE];
+  C v[SH::FE];
   typename A::Acc nacc;
   typename A::Full facc;
 #pragma unroll
-  for (int m = 0; m < SH::XE; ++m) {
-    const int64_t idx = base + (t + m * SH::XT) * S;
+  for (int m = 0; m < SH::FE; ++m) {
+    const int64_t idx = base + (t + m * SH::FT) * S;
     C x = src[idx];
     if (scaled) x = cscale(x, s);
     v[m] = x;
@@ -1696,14 +1706,14 @@ k_forward_x(const typename A::C* src, typename A::C* W, typename A::C* psi_out, 
   }
   if (psi_out) {
 #pragma unroll
-    for (int m = 0; m < SH::XE; ++m) psi_out[base + (t + m * SH::XT) * S] = v[m];
+    for (int m = 0; m < SH::FE; ++m) psi_out[base + (t + m * SH::FT) * S] = v[m];
   }
-  using AT = AccTile<C, SH::XCOLS, SH::XT>;
+  using AT = AccTile<C, SH::XCOLS, SH::FT>;
   __shared__ int mxs[A::id == 0 ? AT::MAXN : 1];
   AT acc{sm, col, col, mxs};
-  fft_line<A, N, -1, AT, false, SH::XR>(v, t, tw, acc);
+  fft_line<A, N, -1, AT, false, SH::FR>(v, t, tw, acc);
 #pragma unroll
-  for (int m = 0; m < SH::XE; ++m) W[base + (t + m * SH::XT) * S] = v[m];
+  for (int m = 0; m < SH::FE; ++m) W[base + (t + m * SH::FT) * S] = v[m];
   if constexpr (STATS == STATS_NORM) norm_reduce_store<A>(nacc, part);
   if constexpr (STATS == STATS_FULL) full_store<A>(facc, part);
 }

@@ -47,7 +47,7 @@ cudaError_t Launch<A, N>::forward_x(const LaunchArgs& a, int* nblocks) {
   const int grid = (int)((int64_t)N * N / SH::XCOLS);
   auto go = [&](auto kern) {
     ensure_smem(kern, smem);
-    pdl_launch(kern, grid, SH::XTHREADS, smem, a.stream, (const C*)a.src, (C*)a.W, (C*)a.psi_out, (const VT*)a.V,
+    pdl_launch(kern, grid, SH::FTHREADS, smem, a.stream, (const C*)a.src, (C*)a.W, (C*)a.psi_out, (const VT*)a.V,
                a.scale, a.scale_f, (const C*)a.tw, a.part);
   };
   if (a.stats == STATS_FULL) go(k_forward_x<A, N, STATS_FULL>);
