@@ -538,7 +538,7 @@ struct qfd_plan_s {
   float2* tw32 = nullptr;
   dfc* twdf = nullptr;
   double* ktab64 = nullptr;
-  void* ttab = nullptr;      // T(k)/N^3 of an octant, FP64 or double-float (16-byte plans of the FFT terms)
+  void* ttab = nullptr;      // T(k)/N^3 of an octant, in ktab64's or ktabdf's allocation (16-byte plans of the FFT terms)
   float* ktab32 = nullptr;
   df* ktabdf = nullptr;
   double* partA = nullptr;
@@ -1734,9 +1734,9 @@ qfd_status qfd_plan(const qfd_params* params, qfd_plan_t* out) {
       {(void**)&pl->tw64, (size_t)4 * n * sizeof(double2)},  // plain twiddles, the scaled block, the fixed-point ones
       {(void**)&pl->tw32, (size_t)n * sizeof(float2)},
       {(void**)&pl->twdf, (size_t)n * sizeof(dfc)},
-      {(void**)&pl->ktab64, (size_t)n * sizeof(double)},
+      {(void**)&pl->ktab64, (size_t)n * sizeof(double) + (pl->arith16 == 0 ? ttab_bytes(p) : 0)},
       {(void**)&pl->ktab32, (size_t)n * sizeof(float)},
-      {(void**)&pl->ktabdf, (size_t)n * sizeof(df)},
+      {(void**)&pl->ktabdf, (size_t)n * sizeof(df) + (pl->arith16 == 2 ? ttab_bytes(p) : 0)},
       {(void**)&pl->partA, (size_t)2 * npart * sizeof(double)},
       {(void**)&pl->partC, (size_t)npart * sizeof(double)},
       {(void**)&pl->partG, (size_t)2 * MAX_LOWER * npart * sizeof(double)},
@@ -1747,7 +1747,6 @@ qfd_status qfd_plan(const qfd_params* params, qfd_plan_t* out) {
   };
   if (uses16(p.precision)) allocs.push_back({(void**)&pl->psi16, (size_t)(p.nstates + 1) * n3 * 16});
   if (uses32(p.precision)) allocs.push_back({(void**)&pl->psi32, (size_t)(p.nstates + 1) * n3 * sizeof(float2)});
-  if (ttab_bytes(p)) allocs.push_back({(void**)&pl->ttab, ttab_bytes(p)});
   if (needs_coef16(p)) allocs.push_back({(void**)&pl->coef16, (size_t)n3 * 16});
   if (needs_coef32(p)) allocs.push_back({(void**)&pl->coef32, (size_t)n3 * sizeof(float2)});
   if (needs_v32(p)) allocs.push_back({(void**)&pl->V32, (size_t)n3 * sizeof(float)});
@@ -1780,8 +1779,10 @@ qfd_status qfd_plan(const qfd_params* params, qfd_plan_t* out) {
     kt32[e] = (float)ktab[e];
     ktdf[e] = host_split(ktab[e]);
   }
-  scaled_twiddle_table(n, tw.data(), tw.data() + n);
-  fixed_twiddle_table(n, tw.data() + 3 * n);
+  if (uses16(p.precision) && pl->arith16 == 0) {
+    scaled_twiddle_table(n, tw.data(), tw.data() + n);
+    fixed_twiddle_table(n, tw.data() + 3 * n);
+  }
   bool ok = cudaMemcpy(pl->tw64, tw.data(), 4 * n * sizeof(double2), cudaMemcpyHostToDevice) == cudaSuccess &&
             cudaMemcpy(pl->tw32, tw32.data(), n * sizeof(float2), cudaMemcpyHostToDevice) == cudaSuccess &&
             cudaMemcpy(pl->twdf, twdf.data(), n * sizeof(dfc), cudaMemcpyHostToDevice) == cudaSuccess &&
@@ -1789,12 +1790,15 @@ qfd_status qfd_plan(const qfd_params* params, qfd_plan_t* out) {
             cudaMemcpy(pl->ktab32, kt32.data(), n * sizeof(float), cudaMemcpyHostToDevice) == cudaSuccess &&
             cudaMemcpy(pl->ktabdf, ktdf.data(), n * sizeof(df), cudaMemcpyHostToDevice) == cudaSuccess &&
             cudaMemset(pl->scal, 0, SC_COUNT * sizeof(double)) == cudaSuccess;
-  if (ok && pl->ttab) {
+  if (ok && ttab_bytes(p)) {  // the octant table, after the per-axis one in its allocation
     const int h = (int)n / 2 + 1;
     const int g = grid_for((int64_t)h * h * h);
+    pl->ttab = pl->arith16 == 0 ? (void*)(pl->ktab64 + n) : (void*)(pl->ktabdf + n);
+    // the uploads above are on the default stream, which the plan's does not wait for
+    ok = cudaStreamSynchronize(0) == cudaSuccess;
     if (pl->arith16 == 0) k_kin_octant<F64><<<g, 256, 0, pl->st>>>(pl->ktab64, pl->kin, h, (double*)pl->ttab);
     else k_kin_octant<DF><<<g, 256, 0, pl->st>>>(pl->ktabdf, pl->kin, h, (df*)pl->ttab);
-    ok = cudaGetLastError() == cudaSuccess && cudaStreamSynchronize(pl->st) == cudaSuccess;
+    ok = ok && cudaGetLastError() == cudaSuccess;
   }
   if (!ok) return cleanup_fail(QFD_ERR_CUDA, "table upload failed");
   if (cudaHostAlloc((void**)&pl->hscal, (SC_COUNT + 1) * sizeof(double), cudaHostAllocDefault) != cudaSuccess)
@@ -1812,7 +1816,7 @@ void qfd_destroy(qfd_plan_t pl) {
   if (!pl) return;
   if (pl->st) cudaStreamSynchronize(pl->st);
   void* bufs[] = {pl->psi16, pl->psi32, pl->W,      pl->coef16, pl->coef32, pl->V,     pl->tw64,
-                  pl->tw32,  pl->twdf,  pl->ktab64, pl->ttab, pl->ktab32, pl->ktabdf, pl->partA, pl->partC,
+                  pl->tw32,  pl->twdf,  pl->ktab64, pl->ktab32, pl->ktabdf, pl->partA, pl->partC,
                   pl->partG, pl->scal,  pl->scalf, pl->flag, pl->Vdf, pl->V32, pl->errflag, pl->tmaps};
   for (void* b : bufs)
     if (b) cudaFree(b);

@@ -14,7 +14,7 @@
 
 namespace qfd {
 
-// The scaled twiddles of the complex128 radix-8 stages (scaled_bfly8 in
+// The scaled twiddles of the FP64 radix-8 stages (scaled_bfly8 in
 // qfd_kernels.cuh), built from the plain table tw[e] = exp(-2 pi i e / n):
 // 2 n double2 (forward block, then inverse), each e0 < n / 8 eight double2.
 // The complex128 twiddle table of a lattice is tw followed by this block.
@@ -53,8 +53,9 @@ inline void scaled_twiddle_table(int64_t n, const double2* tw, double2* out) {
 
 // The twiddles of the fixed-point complex128 lines: exp(-2 pi i e / n) in Q61,
 // each part split into balanced limbs h 2^32 + l (l signed), as int4
-// {rl, rh, il, ih}; n entries of 16 bytes after the scaled block.  Angles are
-// reduced to the first octant in integers and evaluated in long double.
+// {rl, rh, il, ih}; n entries of 16 bytes after the scaled block (n is a multiple
+// of 8).  The n / 8 + 1 angles of the first octant are evaluated in long double
+// (in software on Arm: about a microsecond each), the others mirrored from them.
 inline void fixed_twiddle_table(int64_t n, double2* out) {
   using LD = long double;
   const LD pi = 3.14159265358979323846264338327950288L;
@@ -63,11 +64,17 @@ inline void fixed_twiddle_table(int64_t n, double2* out) {
     *l = (int32_t)(uint32_t)(uint64_t)v;
     *h = (int32_t)((v - (int64_t)*l) / ((int64_t)1 << 32));
   };
+  LD co[129], si[129];  // n <= 1024
+  for (int64_t k = 0; k <= n / 8; ++k) {
+    const LD phi = 2 * pi * (LD)k / (LD)n;
+    co[k] = std::cos(phi);
+    si[k] = std::sin(phi);
+  }
   for (int64_t e = 0; e < n; ++e) {
-    const int64_t q = (4 * e) / n, rem = 4 * e - q * n;  // angle pi/2 (q + rem/n)
-    const bool low = 2 * rem <= n;
-    const LD phi = pi / 2 * (LD)(low ? rem : n - rem) / (LD)n;
-    const LD c = low ? std::cos(phi) : std::sin(phi), s = low ? std::sin(phi) : std::cos(phi);
+    const int64_t q = (4 * e) / n, rem = e - q * (n / 4);  // angle pi/2 q + 2 pi rem/n
+    const bool low = 8 * rem <= n;
+    const int64_t k = low ? rem : n / 4 - rem;
+    const LD c = low ? co[k] : si[k], s = low ? si[k] : co[k];
     const LD re[4] = {c, -s, -c, s}, im[4] = {-s, -c, s, c};
     int32_t w[4];
     limbs(re[q], &w[0], &w[1]);
