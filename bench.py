@@ -501,7 +501,7 @@ def c128_solve_cadence(torch, Q, dev, n, steps):
     parity every 10 steps, an energy check every 100): `steps` steps of the
     workload's ground-state solve at lattice size n with no early stop,
     autotuned, timed with CUDA events after 100 untimed steps.  Gives the
-    per-step time for the native FP64 solve estimate (steps x this time)."""
+    per-step time for the complex128 solve estimate (steps x this time)."""
     stream = torch.cuda.current_stream(dev)
     plan = Q.Plan(n, A, MASS, DTAU, KIN, precision="c128", ortho_every=10, check_every=100, max_steps=100, tol=-1,
                   stream=stream.cuda_stream)

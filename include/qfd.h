@@ -68,7 +68,9 @@ typedef enum {
  * terms use periodic boundaries. */
 enum { QFD_KIN_FDTD = 0, QFD_KIN_P2 = 1, QFD_KIN_SIN2 = 2, QFD_KIN_REL = 3 };
 /* Arithmetic of the steps (reductions end in FP64 in all of them):
- *  QFD_C128          complex128 storage, native FP64 arithmetic;
+ *  QFD_C128          complex128 storage; update, T(k) and sums in FP64, the line
+ *                    transforms in 64-bit fixed point scaled per line (their
+ *                    rounding is below that of FP64 butterflies);
  *  QFD_C64           complex64 storage and FP32 arithmetic;
  *  QFD_C64_REFINE    complex64 bulk to tol_bulk, then QFD_C128 steps of the
  *                    same iteration to tol;
@@ -220,8 +222,9 @@ qfd_status qfd_step(qfd_plan_t plan, int state, int64_t nsteps);
  * nsteps steps of Eq. (iter_proced) (Sec. 2.2, with the FFT kinetic terms of
  * Sec. 2.1), i < count, with exactly the operations qfd_step applies to each.
  * Each pass of a step (the y transforms, the z pass with T(k), the update
- * with the x transforms) is one launch over all the lattices; the cadence
- * (projection, deflation, normalisation) runs per plan.  There is no
+ * with the x transforms) is one launch over all the lattices, and so are the
+ * norms of the lattices that only normalise; projections and deflations run
+ * per plan.  There is no
  * counterpart in the paper, whose code steps one lattice.
  *   plans, states  arrays of `count` entries, 1 <= count <= QFD_MAX_BATCH;
  *                  the plans are distinct, have the same n, the same current

@@ -430,7 +430,8 @@ struct DF {
 // 512 times larger.  Measured against a 64-bit transform, ten steps of 512^3
 // noise are off by 8.4e-16 (relative L2) in this form and by 8.6e-16 with the
 // FP64 butterflies.  Measured at 512^3 (FP64 butterflies, then this form): pass
-// A 12.03 and 4.54 ms, a y pass 5.31 and 1.48, the z pass 11.5 and 3.2.  Lines that do not fit (non-finite values, exponents near the ends of the
+// A 12.03 and 4.54 ms, a y pass 5.31 and 1.48, the z pass 11.5 and 3.2 (3.77, 1.27
+// and 2.50 with 1024 threads an SM and T(k) from a table).  Lines that do not fit (non-finite values, exponents near the ends of the
 // FP64 range) take the FP64 transform instead (fft_line).
 struct __align__(16) ic {
   long long x, y;
