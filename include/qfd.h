@@ -296,7 +296,8 @@ qfd_status qfd_snapshot_states(qfd_plan_t plan, int nout, int parity, int64_t sn
  * of half of it at two CTAs per SM, and (complex64, n = 256..1024) the
  * TMA-staged persistent kernel, on the work lattice and the spare state
  * lattice (5 launches each after 2 warm-ups), and keeps the fastest of each
- * for later launches.  Tilings do not change the arithmetic of a line;
+ * for later launches; where the y and z passes also exist as one launch (see
+ * qfd_set_tuning), that is timed too and kept if it beats the separate ones.  Tilings do not change the arithmetic of a line;
  * the radix schedule changes the order of the operations of a transform.
  * Results agree to rounding whatever is chosen (complex128 / complex64
  * kernels may also differ in where the compiler fuses a multiply-add;
