@@ -70,7 +70,8 @@ enum { QFD_KIN_FDTD = 0, QFD_KIN_P2 = 1, QFD_KIN_SIN2 = 2, QFD_KIN_REL = 3 };
 /* Arithmetic of the steps (reductions end in FP64 in all of them):
  *  QFD_C128          complex128 storage; update, T(k) and sums in FP64, the line
  *                    transforms in 64-bit fixed point scaled per line (their
- *                    rounding is below that of FP64 butterflies);
+ *                    error is about that of FP64 butterflies on lines with
+ *                    one high peak, and smaller on others);
  *  QFD_C64           complex64 storage and FP32 arithmetic;
  *  QFD_C64_REFINE    complex64 bulk to tol_bulk, then QFD_C128 steps of the
  *                    same iteration to tol;

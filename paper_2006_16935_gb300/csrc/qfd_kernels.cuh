@@ -422,17 +422,24 @@ struct DF {
 //
 // A line (one column of a tile, or one z line) is scaled by the exponent E of
 // its largest component: v = x 2^(1081 - E), so |v| < 2^59 (2^58 for N = 96,
-// 192).  A radix-8 butterfly adds at most 3.5 bits (components stay below
-// 2^62.5), and the twiddles, held in Q61, give the product over 8, so every stage
-// starts below 2^59.5 again; the result is v 8^(S-1) 2^(E - 1081) with S stages.
-// Bits are dropped only where the transform has grown: the quantum of the last
-// stage is 2^-53 of the largest input for N = 512, against outputs that may be
-// 512 times larger.  Measured against a 64-bit transform, ten steps of 512^3
-// noise are off by 8.4e-16 (relative L2) in this form and by 8.6e-16 with the
-// FP64 butterflies.  Measured at 512^3 (FP64 butterflies, then this form): pass
+// 192) and the modulus stays below 2^59.5 (2^58.5).  A radix-r stage multiplies the
+// modulus by at most r, and the twiddles, held in Q61, give the product over the
+// radix of the stage that they lead into, so every stage ends below 2^62.5; the
+// result is v N / r0 2^(E - 1081) with r0 the first radix.  Bits are dropped only
+// where the transform may have grown: the last quantum is N / r0 2^-59 of 2^E, 2^-53 for
+// N = 512 and 2^-52 for 1024, or 2^-55 there where the values leave room (fx_spare).
+// Relative L2 error of one line against
+// extended precision, in 1e-16 (FP64 butterflies in parentheses), for one site / a broad
+// state's spectrum / a site on a floor of noise: N = 96 0.4 (0.6), 0.6 (1.5), 0.7 (1.3);
+// 192 0.5 (0.7), 0.8 (1.5), 1.1 (1.4); 256 0.6 (1.2), 0.7 (1.6), 1.1 (1.7); 512 0.7 (1.2),
+// 1.3 (1.7), 1.9 (1.8); 1024 0.5 (1.4), 1.0 (1.8), 1.5 (1.9); noise 0.5 (1.8) throughout.
+// With every product over 8 it was 4.2, 4.1 and 6.1 at 1024.
+// Measured at 512^3 (FP64 butterflies, then this form): pass
 // A 12.03 and 4.54 ms, a y pass 5.31 and 1.48, the z pass 11.5 and 3.2 (3.77, 1.27
-// and 2.50 with 1024 threads an SM and T(k) from a table).  Lines that do not fit (non-finite values, exponents near the ends of the
-// FP64 range) take the FP64 transform instead (fft_line).
+// and 2.50 with 1024 threads an SM and T(k) from a table).  Lines that do not fit
+// (non-finite values, exponents near the ends of the FP64 range) take the FP64
+// transform instead (fft_line).
+__host__ __device__ constexpr int ilog2c(int n) { return n <= 1 ? 0 : 1 + ilog2c(n / 2); }
 struct __align__(16) ic {
   long long x, y;
 };
@@ -461,14 +468,17 @@ __device__ __forceinline__ long long mul_r3(long long v) { return v - mulhi_c(v,
 template <int DIR> __device__ __forceinline__ ic mul_w8(ic a) {
   return DIR > 0 ? ic{mul_r2(a.x - a.y), mul_r2(a.x + a.y)} : ic{mul_r2(a.x + a.y), mul_r2(a.y - a.x)};
 }
-// a w / 8 (DIR < 0) or a conj(w) / 8, rounded
-template <int DIR> __device__ __forceinline__ ic mul_itw(ic a, itw w) {
+// a w / RAD (DIR < 0) or a conj(w) / RAD, rounded, RAD = 2, 4 or 8
+template <int DIR, int RAD> __device__ __forceinline__ ic mul_itw(ic a, itw w) {
+  constexpr int D = 3 - ilog2c(RAD);
   const sp x = limbs(a.x), y = limbs(a.y);
   const int il = DIR < 0 ? w.il : -w.il, ih = DIR < 0 ? w.ih : -w.ih;
-  const long long h = 1ll << 31;
+  const long long h = 1ll << (31 - D);
   const long long mr = mw(y.l, -ih, mw(y.h, -il, mw(x.l, w.rh, mw(x.h, w.rl, h))));
   const long long mi = mw(y.l, w.rh, mw(y.h, w.rl, mw(x.l, ih, mw(x.h, il, h))));
-  return ic{mw(y.h, -ih, mw(x.h, w.rh, mr >> 32)), mw(y.h, w.rh, mw(x.h, ih, mi >> 32))};
+  if constexpr (D == 0) return ic{mw(y.h, -ih, mw(x.h, w.rh, mr >> 32)), mw(y.h, w.rh, mw(x.h, ih, mi >> 32))};
+  return ic{(mw(y.h, -ih, mw(x.h, w.rh, 0)) << D) + (mr >> (32 - D)),
+            (mw(y.h, w.rh, mw(x.h, ih, 0)) << D) + (mi >> (32 - D))};
 }
 // A double as v 2^(1081 - E) (bits below the quantum cut), its exponent field at most E.
 template <int K> __device__ __forceinline__ long long fx_in(double d, int E) {
@@ -485,6 +495,21 @@ __device__ __forceinline__ double fx_out(long long v, int k) {
   const int h = __double2hiint(f);
   return __hiloint2double(h ? h + (k << 20) : 0, __double2loint(f));
 }
+// The last stage's outputs go to doubles one by one, so a thread whose inputs are all
+// below 2^57 (peaked lines; broad ones stay above) scales them up by 8 before their
+// product over 8, which would else set the error.  Returns the bits.  For lines of
+// more than three stages (1024, a step 95.5 -> 97 ms); at 512, where these lines are
+// no worse than in FP64 without it, it costs 4.5% of a step.
+template <int E> __device__ __forceinline__ int fx_spare(ic (&v)[E]) {
+  unsigned m = 0;
+#pragma unroll
+  for (int j = 0; j < E; ++j)
+    m |= (unsigned)((int)(v[j].x >> 32) + (1 << 25)) | (unsigned)((int)(v[j].y >> 32) + (1 << 25));
+  if (m >= 1u << 26) return 0;
+#pragma unroll
+  for (int j = 0; j < E; ++j) v[j] = ic{v[j].x << 3, v[j].y << 3};
+  return 3;
+}
 struct X64 {  // the transform policy of the fixed-point lines
   using C = ic;
   static constexpr int id = 3;
@@ -492,7 +517,6 @@ struct X64 {  // the transform policy of the fixed-point lines
 constexpr int FX_E_MIN = 64, FX_E_MAX = 1960;  // exponent fields of a line that runs in fixed point
 
 // ============================================================ FFT planning
-__host__ __device__ constexpr int ilog2c(int n) { return n <= 1 ? 0 : 1 + ilog2c(n / 2); }
 
 // E elements per thread and the radix schedule of a length-N transform.
 // Schedule R = 0:
@@ -517,13 +541,17 @@ template <int N, int R = 0> struct FftPlan {
   static constexpr int P = ilog2c(R3 ? N / 12 : N);
   static constexpr int Q = R3 ? P / 2 : P / 3;
   static constexpr int REM = R3 ? P % 2 : P % 3;
+  static constexpr bool SHORT2 = R == 3 && !R3 && REM != 0 && Q > 2;  // the short stage second
   static constexpr int S = E16 ? (P2 > 8 ? 3 : 2) : TWO ? 2 : (R3 ? 1 + Q + REM : Q + (REM ? 1 : 0));
   __host__ __device__ static constexpr int radix(int i) {
     return E16 ? (i == 0 ? 16 : i == 1 ? (N < 256 ? N / 16 : 16) : N / 256)
-           : TWO ? (i == 0 ? E : N / E) : R3 ? (i == 0 ? 12 : (i <= Q ? 4 : 2)) : (i < Q ? 8 : (REM == 1 ? 2 : 4));
+           : TWO ? (i == 0 ? E : N / E) : R3 ? (i == 0 ? 12 : (i <= Q ? 4 : 2)) : (i == (SHORT2 ? 1 : Q) ? (REM == 1 ? 2 : 4) : 8);
   }
   __host__ __device__ static constexpr int ns(int i) { return i == 0 ? 1 : ns(i - 1) * radix(i - 1); }
 };
+
+// Schedule R = 3 (the fixed-point lines): as R = 0, but with more than three stages
+// the short one comes second (8, 2, 8, 8 for 1024), so that the last is of radix 8.
 
 // Complex constants in the representation of C.
 __device__ __forceinline__ double2 cconst(double re, double im, double2) { return double2{re, im}; }
@@ -784,12 +812,15 @@ template <> struct TwOf<X64> {
 // instead of table loads (complex64 only; used where the table loads compete
 // with the shared-memory exchanges for the L1 pipe: the z-pass and the
 // inverse y pass).
+// Returns the bits by which a fixed-point last stage has scaled its line up (fx_spare).
 template <class A, int N, int R, int RAD, int NS, int DIR, bool LAST, bool TWC = false>
-__device__ __forceinline__ void stage_compute(typename A::C (&v)[FftPlan<N, R>::E], int t,
+__device__ __forceinline__ int stage_compute(typename A::C (&v)[FftPlan<N, R>::E], int t,
                                               const typename TwOf<A>::type* __restrict__ tw) {
   using C = typename A::C;
   constexpr int E = FftPlan<N, R>::E;
   constexpr int NB = E / RAD;
+  int up = 0;
+  if constexpr (A::id == 3 && LAST && FftPlan<N, R>::S > 3) up = fx_spare<E>(v);
   // complex128 twiddled radix-8 stages: the scaled-twiddle butterfly
   constexpr bool SCALED = A::id == 0 && RAD == 8 && NS > 1 && R == 0;
 #pragma unroll
@@ -808,13 +839,13 @@ __device__ __forceinline__ void stage_compute(typename A::C (&v)[FftPlan<N, R>::
       const int b = t + u * (N / E);
       const int e0 = (b % NS) * (N / (NS * RAD));
       if constexpr (A::id == 3) {
-        // the product over 8 (see the fixed-point section), r = 0 included
+        // the product over RAD (see the fixed-point section), r = 0 included
 #pragma unroll
         for (int r = 1; r < RAD; ++r) {
           const int4 q = __ldg(reinterpret_cast<const int4*>(tw + e0 * r));
-          x[r] = mul_itw<DIR>(x[r], itw{q.x, q.y, q.z, q.w});
+          x[r] = mul_itw<DIR, RAD>(x[r], itw{q.x, q.y, q.z, q.w});
         }
-        x[0] = ic{(x[0].x + 4) >> 3, (x[0].y + 4) >> 3};
+        x[0] = ic{(x[0].x + RAD / 2) >> ilog2c(RAD), (x[0].y + RAD / 2) >> ilog2c(RAD)};
       } else if constexpr (TWC && A::id == 1) {
         // w = exp(-2 pi i e0 / N) from sincospif, its powers by products
         // (a few ulp of FP32, like the rounding of the transform itself)
@@ -843,6 +874,7 @@ __device__ __forceinline__ void stage_compute(typename A::C (&v)[FftPlan<N, R>::
 #pragma unroll
     for (int r = 0; r < RAD; ++r) v[u + r * NB] = cnorm(x[r]);
   }
+  return up;
 }
 
 // Writes stage outputs to their Stockham positions, then reads the canonical set.
@@ -866,16 +898,18 @@ __device__ __forceinline__ void stage_exchange(C (&v)[FftPlan<N, R>::E], int t, 
 }
 
 template <class A, int N, int R, int DIR, int I, bool TWC, class Acc>
-__device__ __forceinline__ void fft_stages(typename A::C (&v)[FftPlan<N, R>::E], int t,
+__device__ __forceinline__ int fft_stages(typename A::C (&v)[FftPlan<N, R>::E], int t,
                                            const typename TwOf<A>::type* __restrict__ tw, Acc& acc) {
   using PL = FftPlan<N, R>;
   if constexpr (I < PL::S) {
     constexpr int RAD = PL::radix(I);
     constexpr int NS = PL::ns(I);
-    stage_compute<A, N, R, RAD, NS, DIR, I + 1 == PL::S, TWC>(v, t, tw);
-    if constexpr (I + 1 < PL::S) stage_exchange<typename A::C, N, R, RAD, NS>(v, t, acc);
-    fft_stages<A, N, R, DIR, I + 1, TWC>(v, t, tw, acc);
+    const int up = stage_compute<A, N, R, RAD, NS, DIR, I + 1 == PL::S, TWC>(v, t, tw);
+    if constexpr (I + 1 == PL::S) return up;
+    stage_exchange<typename A::C, N, R, RAD, NS>(v, t, acc);
+    return fft_stages<A, N, R, DIR, I + 1, TWC>(v, t, tw, acc);
   }
+  return 0;
 }
 
 // The FP64 transform of the complex128 lines that fixed point does not cover,
@@ -895,7 +929,7 @@ __device__ __noinline__ void fft_line_f64(double2* v, int t, const double2* __re
 template <int N, int DIR, class Acc>
 __device__ __forceinline__ void fft_line_fx(double2 (&v)[FftPlan<N>::E], int t, const double2* __restrict__ tw,
                                             Acc& acc) {
-  using PL = FftPlan<N>;
+  using PL = FftPlan<N, 3>;
   constexpr int K = PL::R3 ? 5 : 6;
   int mx = 0;
 #pragma unroll
@@ -916,8 +950,8 @@ __device__ __forceinline__ void fft_line_fx(double2 (&v)[FftPlan<N>::E], int t, 
 #pragma unroll
   for (int m = 0; m < PL::E; ++m) x[m] = ic{fx_in<K>(v[m].x, E), fx_in<K>(v[m].y, E)};
   auto xacc = acc.template as<ic>();
-  fft_stages<X64, N, 0, DIR, 0, false>(x, t, reinterpret_cast<const itw*>(tw + 3 * N), xacc);
-  const int k = E - 1075 - K + 3 * (PL::S - 1);
+  const int up = fft_stages<X64, N, 3, DIR, 0, false>(x, t, reinterpret_cast<const itw*>(tw + 3 * N), xacc);
+  const int k = E - 1075 - K + ilog2c(N / PL::radix(0)) - up;
 #pragma unroll
   for (int m = 0; m < PL::E; ++m) v[m] = double2{fx_out(x[m].x, k), fx_out(x[m].y, k)};
 }
