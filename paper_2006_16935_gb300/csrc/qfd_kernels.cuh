@@ -1031,12 +1031,14 @@ template <typename C, int PS, int T> struct AccLine {
       asm volatile("bar.sync %0, %1;" ::"r"(1 + line), "r"(T) : "memory");
     }
   }
-  // the lines of a warp (T <= 32) take the same path, else each line its own
+  // the lines of a warp (T <= 32) take the same path, else each line its own; a line of
+  // one thread (n = 8, whose blocks may be eight lanes) has no barrier to share
   __device__ __forceinline__ bool line_max(int& mx, bool odd, int t) {
     if constexpr (T <= 32) {
 #pragma unroll
       for (int o = 1; o < T; o <<= 1) mx = max(mx, __shfl_xor_sync(0xffffffffu, mx, o));
-      return __any_sync(__activemask(), odd);  // (a block of n = 8 planes has eight lanes)
+      if constexpr (T == 1) return odd;
+      return __any_sync(0xffffffffu, odd);
     } else {
       if (odd) mx = 0x7fffffff;
       mx = __reduce_max_sync(0xffffffffu, mx);
@@ -1476,6 +1478,7 @@ __device__ __forceinline__ void zpass_body(typename A::C* W, const typename A::C
 #pragma unroll
   for (int m = 0; m < PL::E; ++m) v[m] = W[line0 * N + t + m * PL::T];
   static_assert(PL::T <= 32 || LINES <= 15, "one named barrier per line");
+  static_assert(PL::T == 1 || PL::T * LINES % 32 == 0, "the lines of a warp vote together");
   constexpr int PS = R == 0 ? SH::PAD_SHIFT : SH::PAD_SHIFT_R1;
   constexpr int LP = R == 0 ? SH::LPAD : SH::LPAD_R1;
   using AL = typename ZLine<A, N, R>::type;
@@ -1561,6 +1564,7 @@ k_plane(const __grid_constant__ BatchZ b) {
   using AT = AccTile<C, PS::COLS, PS::T, SH::LPAD>;
   using AL = AccLine<C, SH::PAD_SHIFT, PS::T>;
   constexpr int E = FftPlan<N>::E, TT = PS::T;
+  static_assert(TT == 1 || PS::THREADS % 32 == 0, "the lines of a warp vote together");
   extern __shared__ __align__(16) unsigned char smraw[];
   C* sm = reinterpret_cast<C*>(smraw);
   __shared__ int mxs[A::id == 0 ? AT::MAXN : 1];

@@ -89,3 +89,11 @@ def test_lines_outside_the_fixed_point_range_512(qfdlib):
     psi[3, 4, 5] = float("nan")
     assert not bool(torch.isfinite(torch.view_as_real(step(n, psi))).any())
     torch.cuda.empty_cache()
+
+
+@pytest.mark.parametrize("n", [8, 16, 32, 64, 128, 256])
+def test_lines_of_different_kinds_in_one_warp(qfdlib, n):
+    # constant along y: of the z lines of a warp one holds all of the state, below the
+    # fixed-point range, and the others are zero
+    psi = state(n, "noise")[:, :1, :].expand(n, n, n).contiguous() * 2.0 ** -970
+    assert rel(step(n, psi) * 2.0 ** 970, reference(psi * 2.0 ** 970)) < TOL
