@@ -414,15 +414,18 @@ qfd_status qfd_fma_rate(int fp64, double* tflops);
 qfd_status qfd_energy_noalloc(const double* psi, const double* V, int64_t n, double a, double mass, int kinetic,
                               int rest_mass, void* stream, double* E, double* norm2);
 
-/* Device bytes a plan with these parameters allocates (used for admission by
- * budget). */
+/* Device bytes a plan with these parameters needs (used for admission by
+ * budget).  A 16-byte plan of the FFT terms takes about n^3 bytes more, a table
+ * of T(k), where that leaves room for another such plan; without the table the
+ * results are the same. */
 size_t qfd_plan_bytes(const qfd_params* params);
 
 /* ------------------------------------------------------------- server ----
  * Continuous batching of solve requests (a serving form of the method; the
  * paper has a single solve per run).  Requests wait in FIFO order and are
  * admitted while the device bytes of the admitted requests (qfd_plan_bytes)
- * stay within hbm_budget_bytes; each admitted request owns a plan on its own
+ * stay within hbm_budget_bytes (their tables of T(k) take what is left of it, and
+ * are given up for a request that needs the room); each admitted request owns a plan on its own
  * stream (priority rising as the lattice shrinks), so requests overlap on the
  * device and each advances at its own pace.  qfd_server_poll admits what
  * fits, queues one period (check_every steps and an energy check, exactly as

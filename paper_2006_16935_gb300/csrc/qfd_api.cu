@@ -538,12 +538,11 @@ struct qfd_plan_s {
   float2* tw32 = nullptr;
   dfc* twdf = nullptr;
   double* ktab64 = nullptr;
-  void* ttab = nullptr;      // T(k)/N^3 of an octant, in ktab64's or ktabdf's allocation (16-byte plans of the FFT terms)
+  void* ttab = nullptr;      // T(k)/N^3 of an octant (16-byte plans of the FFT terms, where there is room), or null
   float* ktab32 = nullptr;
   df* ktabdf = nullptr;
   double* partA = nullptr;
   double* partC = nullptr;
-  double* partG = nullptr;
   int nA = 0, nC = 0;
   double* scal = nullptr;
   float* scalf = nullptr;  // the normalisation factor in FP32 and double-float form
@@ -876,9 +875,9 @@ qfd_status cadence(qfd_plan_t pl, int s, int check) {
     a.offgrid = pl->p.centre == QFD_CENTRE_OFFGRID;
     a.sums = pl->scal + SC_SUMS;
     if (s > 0) {
-      a.part = pl->partG;
+      a.part = pl->partA;
       QFD_RUN(PASS_GS_DOTS, launch_gs_dots<A>(a, GS_BLOCKS));
-      if ((r = finalize(pl, pl->partG, 2 * s, GS_BLOCKS, OP_SUMS)) != QFD_OK) return r;
+      if ((r = finalize(pl, pl->partA, 2 * s, GS_BLOCKS, OP_SUMS)) != QFD_OK) return r;
     }
     a.part = pl->partA;
     a.stats = check ? STATS_FULL : STATS_NORM;
@@ -1349,19 +1348,37 @@ size_t ttab_bytes(const qfd_params& p) {
 }
 bool needs_coef32(const qfd_params& p) { return uses32(p.precision) && p.kinetic == 0; }
 bool needs_v32(const qfd_params& p) { return uses32(p.precision) && p.kinetic != 0; }
-// Device bytes a plan with these parameters allocates (lattices, tables, partials).
+// Per-CTA partials a plan's own arithmetics take.
+int plan_partials(const qfd_params& p) {
+  int m = GS_BLOCKS;
+  if (uses32(p.precision)) m = std::max(m, max_partials<F32>(p.n));
+  if (uses16(p.precision))
+    m = std::max(m, arith16_of(p.precision) == 0 ? max_partials<F64>(p.n) : max_partials<DF>(p.n));
+  return m;
+}
+// The array of the passes' partials, which the per-CTA sums of the overlap and observable
+// kernels share: each is reduced by the launch after the one that writes it.  (k_gs_dots
+// writes the 2 K sums of its instance.)
+size_t partA_entries(const qfd_params& p) {
+  return std::max((size_t)2 * plan_partials(p), (size_t)(p.nstates <= 5 ? NOBS : 2 * MAX_LOWER) * GS_BLOCKS);
+}
+// complex128 twiddles: plain, the scaled block, the fixed-point ones
+int64_t tw64_entries(const qfd_params& p) { return (uses16(p.precision) && arith16_of(p.precision) == 0 ? 4 : 3) * p.n; }
+// double-float twiddles: those plans only
+int64_t twdf_entries(const qfd_params& p) { return uses16(p.precision) && arith16_of(p.precision) == 0 ? 0 : p.n; }
+// Device bytes a plan with these parameters needs (lattices, tables, partials).  The table
+// of T(k) (ttab_bytes) comes on top where there is room for it.
 size_t plan_device_bytes(const qfd_params& p) {
   const size_t n = (size_t)p.n, n3 = n * n * n;
-  const size_t npart = (size_t)std::max(
-      std::max(std::max(max_partials<F64>(p.n), max_partials<F32>(p.n)), max_partials<DF>(p.n)), GS_BLOCKS);
-  size_t b = n3 * 16 + n3 * 8 + n * (64 + 8 + 16 + 8 + 4 + 8) + npart * 8 * (3 + 2 * MAX_LOWER) + 1024;
+  size_t b = n3 * 16 + n3 * 8 + (size_t)(tw64_entries(p) + twdf_entries(p)) * 16 + n * (8 + 8 + 4 + 8) +
+             ((size_t)plan_partials(p) + partA_entries(p)) * 8 + 1024;
   if (uses16(p.precision)) b += (size_t)(p.nstates + 1) * n3 * 16;
   if (uses32(p.precision)) b += (size_t)(p.nstates + 1) * n3 * 8;
   if (needs_coef16(p)) b += n3 * 16;
   if (needs_coef32(p)) b += n3 * 8;
   if (needs_v32(p)) b += n3 * sizeof(float);
   if (uses_vdf(p.precision)) b += n3 * sizeof(df);
-  return b + ttab_bytes(p);
+  return b;
 }
 bool uses32(int precision) {
   return precision == QFD_C64 || precision == QFD_C64_REFINE || precision == QFD_C64_REFINE_DF;
@@ -1626,7 +1643,12 @@ bool build_tensor_maps(qfd_plan_t pl) {
 // ================================================================ C ABI
 extern "C" {
 
-qfd_status qfd_plan(const qfd_params* params, qfd_plan_t* out) {
+}  // extern "C"
+
+// qfd_plan; the table of T(k) is taken if it leaves `reserve` bytes of the device free
+// (a small one, or with reserve 0: if its allocation succeeds).
+constexpr size_t NO_TTAB = ~(size_t)0;
+static qfd_status make_plan(const qfd_params* params, qfd_plan_t* out, size_t reserve) {
   if (out) *out = nullptr;
   if (!params || !out) {
     g_create_error = "null argument";
@@ -1722,8 +1744,7 @@ qfd_status qfd_plan(const qfd_params* params, qfd_plan_t* out) {
     pl->own_stream = true;
   }
   const int64_t n3 = pl->n3;
-  const int npart =
-      std::max(std::max(std::max(max_partials<F64>(n), max_partials<F32>(n)), max_partials<DF>(n)), GS_BLOCKS);
+  const int npart = plan_partials(p);
   struct Alloc {
     void** ptr;
     size_t bytes;
@@ -1731,20 +1752,19 @@ qfd_status qfd_plan(const qfd_params* params, qfd_plan_t* out) {
   std::vector<Alloc> allocs = {
       {(void**)&pl->W, (size_t)n3 * 16},
       {(void**)&pl->V, (size_t)n3 * sizeof(double)},
-      {(void**)&pl->tw64, (size_t)4 * n * sizeof(double2)},  // plain twiddles, the scaled block, the fixed-point ones
+      {(void**)&pl->tw64, (size_t)tw64_entries(p) * sizeof(double2)},
       {(void**)&pl->tw32, (size_t)n * sizeof(float2)},
-      {(void**)&pl->twdf, (size_t)n * sizeof(dfc)},
-      {(void**)&pl->ktab64, (size_t)n * sizeof(double) + (pl->arith16 == 0 ? ttab_bytes(p) : 0)},
+      {(void**)&pl->ktab64, (size_t)n * sizeof(double)},
       {(void**)&pl->ktab32, (size_t)n * sizeof(float)},
-      {(void**)&pl->ktabdf, (size_t)n * sizeof(df) + (pl->arith16 == 2 ? ttab_bytes(p) : 0)},
-      {(void**)&pl->partA, (size_t)2 * npart * sizeof(double)},
+      {(void**)&pl->ktabdf, (size_t)n * sizeof(df)},
+      {(void**)&pl->partA, partA_entries(p) * sizeof(double)},
       {(void**)&pl->partC, (size_t)npart * sizeof(double)},
-      {(void**)&pl->partG, (size_t)2 * MAX_LOWER * npart * sizeof(double)},
       {(void**)&pl->scal, SC_COUNT * sizeof(double)},
       {(void**)&pl->scalf, 16 * sizeof(float)},
       {(void**)&pl->flag, sizeof(int)},
       {(void**)&pl->errflag, sizeof(int)},
   };
+  if (twdf_entries(p)) allocs.push_back({(void**)&pl->twdf, (size_t)twdf_entries(p) * sizeof(dfc)});
   if (uses16(p.precision)) allocs.push_back({(void**)&pl->psi16, (size_t)(p.nstates + 1) * n3 * 16});
   if (uses32(p.precision)) allocs.push_back({(void**)&pl->psi32, (size_t)(p.nstates + 1) * n3 * sizeof(float2)});
   if (needs_coef16(p)) allocs.push_back({(void**)&pl->coef16, (size_t)n3 * 16});
@@ -1757,6 +1777,15 @@ qfd_status qfd_plan(const qfd_params* params, qfd_plan_t* out) {
       char buf[128];
       snprintf(buf, sizeof(buf), "cudaMalloc of %zu bytes failed", a.bytes);
       return cleanup_fail(QFD_ERR_OOM, buf);
+    }
+  }
+  if (ttab_bytes(p) && reserve != NO_TTAB) {
+    size_t free_b = 0, total_b = 0;
+    const bool room = ttab_bytes(p) < ((size_t)2 << 20) || reserve == 0 ||
+                      (cudaMemGetInfo(&free_b, &total_b) == cudaSuccess && free_b >= reserve + ttab_bytes(p));
+    if (!room || cudaMalloc(&pl->ttab, ttab_bytes(p)) != cudaSuccess) {
+      cudaGetLastError();
+      pl->ttab = nullptr;  // the z pass forms T(k) itself
     }
   }
   for (int j = 0; j < p.nstates; ++j) {
@@ -1783,17 +1812,17 @@ qfd_status qfd_plan(const qfd_params* params, qfd_plan_t* out) {
     scaled_twiddle_table(n, tw.data(), tw.data() + n);
     fixed_twiddle_table(n, tw.data() + 3 * n);
   }
-  bool ok = cudaMemcpy(pl->tw64, tw.data(), 4 * n * sizeof(double2), cudaMemcpyHostToDevice) == cudaSuccess &&
+  bool ok = cudaMemcpy(pl->tw64, tw.data(), tw64_entries(p) * sizeof(double2), cudaMemcpyHostToDevice) == cudaSuccess &&
             cudaMemcpy(pl->tw32, tw32.data(), n * sizeof(float2), cudaMemcpyHostToDevice) == cudaSuccess &&
-            cudaMemcpy(pl->twdf, twdf.data(), n * sizeof(dfc), cudaMemcpyHostToDevice) == cudaSuccess &&
+            (!pl->twdf ||
+             cudaMemcpy(pl->twdf, twdf.data(), n * sizeof(dfc), cudaMemcpyHostToDevice) == cudaSuccess) &&
             cudaMemcpy(pl->ktab64, ktab.data(), n * sizeof(double), cudaMemcpyHostToDevice) == cudaSuccess &&
             cudaMemcpy(pl->ktab32, kt32.data(), n * sizeof(float), cudaMemcpyHostToDevice) == cudaSuccess &&
             cudaMemcpy(pl->ktabdf, ktdf.data(), n * sizeof(df), cudaMemcpyHostToDevice) == cudaSuccess &&
             cudaMemset(pl->scal, 0, SC_COUNT * sizeof(double)) == cudaSuccess;
-  if (ok && ttab_bytes(p)) {  // the octant table, after the per-axis one in its allocation
+  if (ok && pl->ttab) {
     const int h = (int)n / 2 + 1;
     const int g = grid_for((int64_t)h * h * h);
-    pl->ttab = pl->arith16 == 0 ? (void*)(pl->ktab64 + n) : (void*)(pl->ktabdf + n);
     // the uploads above are on the default stream, which the plan's does not wait for
     ok = cudaStreamSynchronize(0) == cudaSuccess;
     if (pl->arith16 == 0) k_kin_octant<F64><<<g, 256, 0, pl->st>>>(pl->ktab64, pl->kin, h, (double*)pl->ttab);
@@ -1812,12 +1841,19 @@ qfd_status qfd_plan(const qfd_params* params, qfd_plan_t* out) {
   return QFD_OK;
 }
 
+extern "C" {
+
+// A plan leaves room for another like it before it takes the table.
+qfd_status qfd_plan(const qfd_params* params, qfd_plan_t* out) {
+  return make_plan(params, out, params ? plan_device_bytes(*params) : 0);
+}
+
 void qfd_destroy(qfd_plan_t pl) {
   if (!pl) return;
   if (pl->st) cudaStreamSynchronize(pl->st);
   void* bufs[] = {pl->psi16, pl->psi32, pl->W,      pl->coef16, pl->coef32, pl->V,     pl->tw64,
                   pl->tw32,  pl->twdf,  pl->ktab64, pl->ktab32, pl->ktabdf, pl->partA, pl->partC,
-                  pl->partG, pl->scal,  pl->scalf, pl->flag, pl->Vdf, pl->V32, pl->errflag, pl->tmaps};
+                  pl->scal,  pl->scalf, pl->flag, pl->Vdf, pl->V32, pl->errflag, pl->tmaps, pl->ttab};
   for (void* b : bufs)
     if (b) cudaFree(b);
   if (pl->hscal) cudaFreeHost(pl->hscal);
@@ -1868,8 +1904,8 @@ qfd_status qfd_add_random_field(qfd_plan_t pl, uint64_t seed, double corr, doubl
   QFD_RUN(PASS_OTHER, (k_grf_conv<<<g, 256, 0, pl->st>>>(f0, f1, Lat{pl->p.n, pl->lg}, 0, taps), cudaGetLastError()));
   QFD_RUN(PASS_OTHER, (k_grf_conv<<<g, 256, 0, pl->st>>>(f1, f0, Lat{pl->p.n, pl->lg}, 1, taps), cudaGetLastError()));
   QFD_RUN(PASS_OTHER, (k_grf_conv<<<g, 256, 0, pl->st>>>(f0, f1, Lat{pl->p.n, pl->lg}, 2, taps), cudaGetLastError()));
-  QFD_RUN(PASS_OTHER, (k_grf_moments<<<GS_BLOCKS, 256, 0, pl->st>>>(f1, pl->n3, pl->partG), cudaGetLastError()));
-  qfd_status r = finalize(pl, pl->partG, 2, GS_BLOCKS, OP_SUMS);
+  QFD_RUN(PASS_OTHER, (k_grf_moments<<<GS_BLOCKS, 256, 0, pl->st>>>(f1, pl->n3, pl->partA), cudaGetLastError()));
+  qfd_status r = finalize(pl, pl->partA, 2, GS_BLOCKS, OP_SUMS);
   if (r != QFD_OK) return r;
   QFD_RUN(PASS_OTHER, (k_grf_add<<<g, 256, 0, pl->st>>>(pl->V, f1, pl->n3, pl->scal + SC_SUMS, amplitude),
                        cudaGetLastError()));
@@ -1987,8 +2023,8 @@ qfd_status qfd_observables(qfd_plan_t pl, int s, double min_sep_edge, double* ou
     qfd_status q = materialize<A>(pl, s);
     if (q != QFD_OK) return q;
     QFD_RUN(PASS_OTHER, pdl_launch(k_observables<A>, GS_BLOCKS, 256, 0, pl->st, psi_of<A>(pl, s), lat, offgrid,
-                                   half, pl->partG));
-    return finalize(pl, pl->partG, NOBS, GS_BLOCKS, OP_OBS);
+                                   half, pl->partA));
+    return finalize(pl, pl->partA, NOBS, GS_BLOCKS, OP_OBS);
   });
   if (r != QFD_OK) return r;
   double h[NOBS];
@@ -2477,13 +2513,36 @@ qfd_status server_shapes(qfd_server_t sv, qfd_plan_t pl) {
   return QFD_OK;
 }
 
+// Frees the table of T(k) of an active request (its next periods form T(k) again, with
+// the same values) and drops the captured periods that read it.  Returns the bytes.
+size_t shed_table(qfd_server_t sv, ReqRun* m) {
+  if (!m->plan->ttab) return 0;
+  if (cudaStreamSynchronize(m->st) != cudaSuccess) return 0;  // (reported by the period in flight)
+  cudaFree(m->plan->ttab);
+  m->plan->ttab = nullptr;
+  cudaGraphExec_t& exec = m->cohort ? m->cohort->exec : m->exec;
+  if (exec) cudaGraphExecDestroy(exec);
+  exec = nullptr;
+  const size_t b = ttab_bytes(m->plan->p);
+  m->bytes -= b;
+  sv->used -= b;
+  return b;
+}
+
+// A request is admitted if its lattices fit the budget.  The tables of T(k) only take
+// what the budget leaves, and make way for a request that needs the room.
 qfd_status admit(qfd_server_t sv) {
   while (!sv->waiting.empty()) {
     if (sv->p.max_active > 0 && (int)sv->active.size() >= sv->p.max_active) break;
     ReqRun* m = sv->waiting.front();
     qfd_params prm = request_params(sv, m->req);
     m->bytes = plan_device_bytes(prm);
-    if (sv->used + m->bytes > (size_t)sv->p.hbm_budget_bytes) {
+    const size_t budget = (size_t)sv->p.hbm_budget_bytes;
+    size_t tables = 0;
+    for (ReqRun* q : sv->active) tables += q->plan->ttab ? ttab_bytes(q->plan->p) : 0;
+    if (sv->used + m->bytes > budget && sv->used - tables + m->bytes <= budget)
+      for (size_t i = 0; i < sv->active.size() && sv->used + m->bytes > budget; ++i) shed_table(sv, sv->active[i]);
+    if (sv->used + m->bytes > budget) {
       if (!sv->active.empty()) break;  // wait for memory to free up
       sv->waiting.pop_front();         // can never fit the budget
       finish_request(sv, m, QFD_ERR_OOM);
@@ -2529,7 +2588,14 @@ qfd_status admit(qfd_server_t sv) {
       continue;
     }
     prm.stream = (void*)m->st;
-    qfd_status r = qfd_plan(&prm, &m->plan);
+    const size_t reserve = sv->used + m->bytes + ttab_bytes(prm) <= budget ? 0 : NO_TTAB;
+    qfd_status r = make_plan(&prm, &m->plan, reserve);
+    if (r == QFD_ERR_OOM) {
+      size_t freed = 0;
+      for (ReqRun* q : sv->active) freed += shed_table(sv, q);
+      if (freed) r = make_plan(&prm, &m->plan, reserve);
+    }
+    if (m->plan && m->plan->ttab) m->bytes += ttab_bytes(prm);
     if (r == QFD_ERR_OOM && !sv->active.empty()) {  // retry once memory frees up
       if (m->cohort) {
         auto& mem = m->cohort->members;
