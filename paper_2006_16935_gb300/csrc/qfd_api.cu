@@ -160,8 +160,8 @@ template <class A> __global__ void k_scale_batch(const __grid_constant__ BatchS 
 // T(k)/N^3 for kx, ky, kz < h = N/2 + 1, in the order and with the operations of
 // the z pass.
 template <class A>
-__global__ void k_kin_octant(const typename A::T* __restrict__ ktab, KinParams kp, int h,
-                             typename A::T* __restrict__ out) {
+__global__ void k_kin_octant(const typename A::T* ktab, KinParams kp, int h, typename A::T* __restrict__ out) {
+  pdl_begin();
   const int64_t h3 = (int64_t)h * h * h;
   for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < h3; i += (int64_t)gridDim.x * blockDim.x) {
     const int z = (int)(i % h), y = (int)(i / h % h), x = (int)(i / ((int64_t)h * h));
@@ -597,7 +597,10 @@ qfd_status fail(qfd_plan_t pl, qfd_status s, const std::string& msg) {
 #define QFD_CK(call)                                                                             \
   do {                                                                                           \
     cudaError_t e_ = (call);                                                                     \
-    if (e_ != cudaSuccess) return fail(pl, QFD_ERR_CUDA, std::string(#call) + ": " + cudaGetErrorString(e_)); \
+    if (e_ != cudaSuccess) {                                                                     \
+      cudaGetLastError(); /* reported here, and not again by the next launch check */            \
+      return fail(pl, QFD_ERR_CUDA, std::string(#call) + ": " + cudaGetErrorString(e_));         \
+    }                                                                                            \
   } while (0)
 
 // Launch f() (which returns cudaError_t), bracketed by timing events when enabled.
@@ -1825,9 +1828,10 @@ static qfd_status make_plan(const qfd_params* params, qfd_plan_t* out, size_t re
     const int g = grid_for((int64_t)h * h * h);
     // the uploads above are on the default stream, which the plan's does not wait for
     ok = cudaStreamSynchronize(0) == cudaSuccess;
-    if (pl->arith16 == 0) k_kin_octant<F64><<<g, 256, 0, pl->st>>>(pl->ktab64, pl->kin, h, (double*)pl->ttab);
-    else k_kin_octant<DF><<<g, 256, 0, pl->st>>>(pl->ktabdf, pl->kin, h, (df*)pl->ttab);
-    ok = ok && cudaGetLastError() == cudaSuccess;
+    // (the launch's own status: the last error may be that of an earlier call of the caller's)
+    ok = ok && (pl->arith16 == 0
+                    ? pdl_launch(k_kin_octant<F64>, g, 256, 0, pl->st, pl->ktab64, pl->kin, h, (double*)pl->ttab)
+                    : pdl_launch(k_kin_octant<DF>, g, 256, 0, pl->st, pl->ktabdf, pl->kin, h, (df*)pl->ttab)) == cudaSuccess;
   }
   if (!ok) return cleanup_fail(QFD_ERR_CUDA, "table upload failed");
   if (cudaHostAlloc((void**)&pl->hscal, (SC_COUNT + 1) * sizeof(double), cudaHostAllocDefault) != cudaSuccess)
