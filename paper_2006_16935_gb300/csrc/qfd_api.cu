@@ -1925,17 +1925,44 @@ qfd_status qfd_get_potential(qfd_plan_t pl, double* V, int on_device) {
   return QFD_OK;
 }
 
-// Whether a conversion kernel may read or write the caller's lattice in place:
-// memory of the current device, aligned to a complex128 site.
-static bool direct_lattice(const void* p, int on_device) {
-  if (!on_device || (uintptr_t)p % sizeof(double2) != 0) return false;
-  cudaPointerAttributes at{};
-  int dev = -1;
-  if (cudaPointerGetAttributes(&at, p) != cudaSuccess || cudaGetDevice(&dev) != cudaSuccess) {
-    cudaGetLastError();
-    return false;
-  }
-  return at.type == cudaMemoryTypeDevice && at.device == dev;
+// Bytes from p to the end of the allocation it lies in if that is plain memory of the
+// current device, else 0.  (One driver query for all of it; a 64^3 complex64 call of set,
+// 20 steps and get takes 250 us with or without it.)
+static size_t device_bytes_from(const void* p) {
+  using GetAttributes = CUresult (*)(unsigned, CUpointer_attribute*, void**, CUdeviceptr);
+  static std::once_flag once;
+  static GetAttributes fn = nullptr;
+  std::call_once(once, [] {
+    void* f = nullptr;
+    cudaDriverEntryPointQueryResult q = cudaDriverEntryPointSymbolNotFound;
+    if (cudaGetDriverEntryPointByVersion("cuPointerGetAttributes", &f, 12000, cudaEnableDefault, &q) == cudaSuccess &&
+        q == cudaDriverEntryPointSuccess)
+      fn = reinterpret_cast<GetAttributes>(f);
+    else
+      cudaGetLastError();
+  });
+  unsigned type = 0, managed = 0;
+  int of = -1, dev = -2;
+  CUdeviceptr base = 0;
+  size_t size = 0;
+  CUpointer_attribute at[] = {CU_POINTER_ATTRIBUTE_MEMORY_TYPE, CU_POINTER_ATTRIBUTE_IS_MANAGED,
+                              CU_POINTER_ATTRIBUTE_DEVICE_ORDINAL, CU_POINTER_ATTRIBUTE_RANGE_START_ADDR,
+                              CU_POINTER_ATTRIBUTE_RANGE_SIZE};
+  void* val[] = {&type, &managed, &of, &base, &size};
+  if (!fn || fn(5, at, val, (CUdeviceptr)(uintptr_t)p) != CUDA_SUCCESS || cudaGetDevice(&dev) != cudaSuccess) return 0;
+  return type == CU_MEMORYTYPE_DEVICE && !managed && of == dev ? (size_t)(base + size - (CUdeviceptr)(uintptr_t)p) : 0;
+}
+
+// How a conversion gets at the caller's lattice.  IN_PLACE: the kernel reads or writes it,
+// which no copy checks, so it is memory of the current device, aligned to a complex128
+// site, and the whole lattice lies in its allocation.  STAGED: through W and a copy.
+// TOO_SHORT: an allocation ends inside the lattice and none follows it (the copy refuses
+// that too).
+enum class LatticeAccess { IN_PLACE, STAGED, TOO_SHORT };
+static LatticeAccess lattice_access(const void* p, size_t bytes, int on_device) {
+  const size_t rest = on_device ? device_bytes_from(p) : 0;
+  if (rest > 0 && rest < bytes && device_bytes_from((const char*)p + rest) == 0) return LatticeAccess::TOO_SHORT;
+  return rest >= bytes && (uintptr_t)p % sizeof(double2) == 0 ? LatticeAccess::IN_PLACE : LatticeAccess::STAGED;
 }
 
 qfd_status qfd_set_psi(qfd_plan_t pl, int s, const double* psi, int on_device) {
@@ -1950,7 +1977,9 @@ qfd_status qfd_set_psi(qfd_plan_t pl, int s, const double* psi, int on_device) {
   } else {
     // round into the plan's representation, from the caller's lattice or a copy of it in W
     const double2* src = reinterpret_cast<const double2*>(psi);
-    if (!direct_lattice(psi, on_device)) {
+    const LatticeAccess acc = lattice_access(psi, bytes, on_device);
+    if (acc == LatticeAccess::TOO_SHORT) return fail(pl, QFD_ERR_CUDA, "psi: the allocation ends inside the lattice");
+    if (acc == LatticeAccess::STAGED) {
       QFD_CK(cudaMemcpyAsync(pl->W, psi, bytes, kind, pl->st));
       pl->w_stage = ST_NONE;
       src = pl->W;
@@ -1999,7 +2028,9 @@ qfd_status qfd_get_psi(qfd_plan_t pl, int s, double* out, int on_device) {
       QFD_CK(cudaMemcpyAsync(out, psi_of<A>(pl, s), bytes, kind, pl->st));
     } else {
       // into the caller's lattice, or staged in W
-      const bool direct = direct_lattice(out, on_device);
+      const LatticeAccess acc = lattice_access(out, bytes, on_device);
+      if (acc == LatticeAccess::TOO_SHORT) return fail(pl, QFD_ERR_CUDA, "out: the allocation ends inside the lattice");
+      const bool direct = acc == LatticeAccess::IN_PLACE;
       double2* dst = direct ? reinterpret_cast<double2*>(out) : pl->W;
       QFD_RUN(PASS_OTHER, pdl_launch(k_convert<A, F64>, grid_for(pl->n3), 256, 0, pl->st, psi_of<A>(pl, s), dst, pl->n3));
       if (!direct) {
