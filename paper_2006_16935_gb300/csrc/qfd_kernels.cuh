@@ -808,10 +808,11 @@ template <> struct TwOf<X64> {
 // One Stockham stage on the register-resident canonical set v[m] = x[t + m N/E].
 // Butterfly b = t + u N/E (u < E/RAD) takes x[b + r N/RAD] = v[u + r (E/RAD)],
 // multiplies input r by w_N^{(b mod NS) r N/(NS RAD)}, and applies DFT_RAD.
-// TWC: the twiddles of a stage from one sincospif and products of powers
-// instead of table loads (complex64 only; used where the table loads compete
-// with the shared-memory exchanges for the L1 pipe: the z-pass and the
-// inverse y pass).
+// TWC: the twiddles of a stage from one sincospif (radix 8 and less) or a few
+// table entries (radix 16 and 32) and products, instead of a load each
+// (complex64 only; used where the table loads compete with the shared-memory
+// exchanges for the L1 pipe: the z-pass, the inverse y pass and the two-stage
+// schedule).
 // Returns the bits by which a fixed-point last stage has scaled its line up (fx_spare).
 template <class A, int N, int R, int RAD, int NS, int DIR, bool LAST, bool TWC = false>
 __device__ __forceinline__ int stage_compute(typename A::C (&v)[FftPlan<N, R>::E], int t,
@@ -846,6 +847,32 @@ __device__ __forceinline__ int stage_compute(typename A::C (&v)[FftPlan<N, R>::E
           x[r] = mul_itw<DIR, RAD>(x[r], itw{q.x, q.y, q.z, q.w});
         }
         x[0] = ic{(x[0].x + RAD / 2) >> ilog2c(RAD), (x[0].y + RAD / 2) >> ilog2c(RAD)};
+      } else if constexpr (TWC && A::id == 1 && R == 1) {
+        // the two-stage schedule's radix 16 and 32: w_(4k+q) = w_4k w_q, with w_1, w_2, w_4, w_8 and
+        // w_16 from the table.  All powers from w_1 multiply its rounding error by up to 31: one
+        // step of noise was off by 3.98e-7 / 4.37e-7 / 6.64e-7 at 256^3 / 512^3 / 1024^3; so it is by
+        // 3.33e-7 / 3.70e-7 / 3.93e-7 (radix 8: 3.29e-7 / 3.81e-7 / 3.96e-7; the whole table: 3.15e-7 /
+        // 3.58e-7 / 3.80e-7).  Step times (ms): powers 0.237 / 2.09 / 22.6, this 0.239 / 2.10 / 22.8,
+        // the whole table 0.241 / 2.16 / 23.8, radix 8 0.247 / 2.18 / 25.5.
+        C lo[4], hi[RAD / 4];
+        lo[1] = A::ldtw(&tw[e0]);
+        lo[2] = A::ldtw(&tw[2 * e0]);
+        lo[3] = cmul(lo[1], lo[2]);
+        hi[1] = A::ldtw(&tw[4 * e0]);
+        if constexpr (RAD > 8) {
+          hi[2] = A::ldtw(&tw[8 * e0]);
+          hi[3] = cmul(hi[1], hi[2]);
+        }
+        if constexpr (RAD > 16) {
+          hi[4] = A::ldtw(&tw[16 * e0]);
+#pragma unroll
+          for (int k = 5; k < RAD / 4; ++k) hi[k] = cmul(hi[4], hi[k - 4]);
+        }
+#pragma unroll
+        for (int r = 1; r < RAD; ++r) {
+          const C w = r < 4 ? lo[r] : r % 4 == 0 ? hi[r / 4] : cmul(hi[r / 4], lo[r % 4]);
+          x[r] = DIR < 0 ? cmul(x[r], w) : cmulc(x[r], w);
+        }
       } else if constexpr (TWC && A::id == 1) {
         // w = exp(-2 pi i e0 / N) from sincospif, its powers by products
         // (a few ulp of FP32, like the rounding of the transform itself)
@@ -1409,9 +1436,9 @@ __device__ __forceinline__ void fft_strided_body(typename A::C* W, const typenam
   using AT = AccTile<C, YC, PL::T>;
   __shared__ int mxs[A::id == 0 ? AT::MAXN : 1];
   AT acc{sm, col, col, mxs};
-  // complex64 inverse y pass and the two-stage schedule: computed twiddles
-  // (measured faster there; the forward y pass of schedule 0 is faster with
-  // the table)
+  // complex64 inverse y pass and the two-stage schedule: computed twiddles (TWC;
+  // measured faster there; the forward y pass of schedule 0 is faster with the
+  // table)
   fft_line<A, N, DIR, decltype(acc), (DIR > 0 || R == 1), R>(v, t, tw, acc);
 #pragma unroll
   for (int m = 0; m < PL::E; ++m) W[base + (int64_t)(t + m * PL::T) * stride] = v[m];

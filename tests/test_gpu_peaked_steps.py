@@ -91,7 +91,7 @@ def test_lines_outside_the_fixed_point_range_512(qfdlib):
     torch.cuda.empty_cache()
 
 
-@pytest.mark.parametrize("n", [8, 16, 32, 64, 128, 256])
+@pytest.mark.parametrize("n", [8, 16, 32, 64, 128, 256, 512])
 def test_lines_of_different_kinds_in_one_warp(qfdlib, n):
     # constant along y: of the z lines of a warp one holds all of the state, below the
     # fixed-point range, and the others are zero
