@@ -298,8 +298,9 @@ qfd_status qfd_snapshot_states(qfd_plan_t plan, int nout, int parity, int64_t sn
  * TMA-staged persistent kernel, on the work lattice and the spare state
  * lattice (5 launches each after 2 warm-ups), and keeps the fastest of each
  * for later launches; where the y and z passes also exist as one launch (see
- * qfd_set_tuning), that is timed too and kept if it beats the separate ones.  Tilings do not change the arithmetic of a line;
- * the radix schedule changes the order of the operations of a transform.
+ * qfd_set_tuning), that is timed too and kept if it beats the separate ones.
+ * Tilings do not change the arithmetic of a line; the radix schedule changes
+ * the order of the operations of a transform.
  * Results agree to rounding whatever is chosen (complex128 / complex64
  * kernels may also differ in where the compiler fuses a multiply-add;
  * double-float tilings are bit-identical).  ms_out (NULL or 27 doubles): per
@@ -317,7 +318,8 @@ qfd_status qfd_autotune(qfd_plan_t plan, double* ms_out);
  * persistent pass A.  The two-stage schedule exists for complex64 at
  * n = 128..1024 and the TMA pass A for complex64 at n = 256..1024 (when the
  * plan could build its tensor maps, qfd_has_tma); elsewhere 2 runs the default.
- * With y_variant 0 and z_variant -1 (the defaults) the y and z passes of small
+ * A plan starts with (0, -1, 0), policy 1 at n = 256..1024 with (2, -1, 0).
+ * With y_variant 0 and z_variant -1 the y and z passes of small
  * lattices (complex64 up to n = 128, 16-byte arithmetics up to 32) run as one
  * launch over the planes x = const; any other setting, and the per-pass
  * timing of qfd_timing_enable, runs them separately.

@@ -422,7 +422,9 @@ k_fdtd_update(const typename A::C* psi, typename A::C* __restrict__ out,
   typename A::Full facc;
   // sites per thread unrolled in the stencil loop (measured at 512^3: four for
   // double-float, one for complex64, six for complex128: 256^3 440 us with two,
-  // 364 with four, 340 with six, 345 with eight, and 516 with FP64 sums)
+  // 364 with four, 340 with six, 345 with eight, and 516 with FP64 sums).  The
+  // complex128 form is bound by FP64 issue (pipe 76% busy, ALU 59%, DRAM 32%): ten
+  // operations a site, the two conversions of the sums, 6 psi - s, c and the update.
   constexpr int U = A::id == 1 ? 1 : A::id == 0 ? 6 : 4;
 #pragma unroll U
   for (int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; idx < n3; idx += (int64_t)gridDim.x * blockDim.x) {
@@ -1316,6 +1318,9 @@ qfd_status check_state(qfd_plan_t pl, int s) {
   return QFD_OK;
 }
 
+// The host waits here for V's kernels and copies, k_coef and the plan's own set-up: the
+// step kernels read all of that through the read-only path, which their programmatic
+// wait does not order (pdl_begin).
 qfd_status derive_coefficients(qfd_plan_t pl) {
   QFD_CK(cudaMemsetAsync(pl->flag, 0, sizeof(int), pl->st));
   double2* c64 = (pl->coef16 && pl->arith16 == 0) ? (double2*)pl->coef16 : nullptr;

@@ -46,9 +46,13 @@ namespace qfd {
 // launch without it, 1.4-1.7 us with it.  No kernel releases its successor early
 // (griddepcontrol.launch_dependents): the waiting CTAs then pile up on the SMs
 // that drain first and leave the others idle (96^3 double-float step 77 -> 101 us).
-// Arrays that an earlier kernel of the stream may have written are read through
-// plain pointers (no const __restrict__: the read-only path is not ordered by
-// the wait, and the compiler may move such loads above it).
+// Arrays that the launch just before may have written are read through plain
+// pointers: loads of const __restrict__ arrays (the read-only path) are not ordered
+// by the wait, and the compiler may move them above it.  The arrays read that way
+// (twiddles, kinetic tables, T(k), V and the update coefficients) are never written
+// by the launch just before: plan creation uploads or forms them, and
+// derive_coefficients, which every plan passes before its first step, waits on the
+// host for all of it; qfd_energy_noalloc copies its tables before its first kernel.
 __device__ __forceinline__ void pdl_begin() {
   asm volatile("griddepcontrol.wait;" ::: "memory");
 }
@@ -415,8 +419,8 @@ struct DF {
 
 // ============================================================ fixed point
 // The complex128 line transforms run on 64-bit integers.  GB300 issues two FP64
-// operations a clock and SM, but 128 integer additions and 64 multiply-adds of
-// 32 x 32 + 64 bits: an FP64 butterfly costs about ten times the clocks of the
+// operations a clock and SM, but 118 integer additions and 57 multiply-adds of
+// 32 x 32 + 64 bits (measured): an FP64 butterfly costs about ten times the clocks of the
 // same butterfly in fixed point, and a line of doubles needs no more than 64
 // bits once it is scaled by its largest element.
 //
@@ -434,11 +438,15 @@ struct DF {
 // 192 0.5 (0.7), 0.8 (1.5), 1.1 (1.4); 256 0.6 (1.2), 0.7 (1.6), 1.1 (1.7); 512 0.7 (1.2),
 // 1.3 (1.7), 1.9 (1.8); 1024 0.5 (1.4), 1.0 (1.8), 1.5 (1.9); noise 0.5 (1.8) throughout.
 // With every product over 8 it was 4.2, 4.1 and 6.1 at 1024.
-// Measured at 512^3 (FP64 butterflies, then this form): pass
-// A 12.03 and 4.54 ms, a y pass 5.31 and 1.48, the z pass 11.5 and 3.2 (3.77, 1.27
-// and 2.50 with 1024 threads an SM and T(k) from a table).  Lines that do not fit
-// (non-finite values, exponents near the ends of the FP64 range) take the FP64
-// transform instead (fft_line).
+// Measured at 512^3 (FP64 butterflies, then this form): pass A 12.03 and 4.54 ms, a y
+// pass 5.31 and 1.48, the z pass 11.5 and 3.2 (3.77, 1.27 and 2.50 with 1024 threads an
+// SM and T(k) from a table).  Lines that do not fit (non-finite values, a largest
+// component outside 2^-959 to 2^937) take the FP64 transform instead, with the lines
+// that share their barriers.  A tile decides on its threads' parts: one thread that
+// holds only non-zero values below 2^-959 sends it to FP64, though its line may fit.
+// (Asking for the lines' maxima, known past the barrier, gains 8% of the first step of a
+// state that falls to 1e-290, after which rounding fills the tails, and costs every
+// other step: 32^3 18.8 -> 19.2 us, 512^3 8.82 -> 8.84 ms.)
 __host__ __device__ constexpr int ilog2c(int n) { return n <= 1 ? 0 : 1 + ilog2c(n / 2); }
 struct __align__(16) ic {
   long long x, y;
@@ -526,32 +534,31 @@ constexpr int FX_E_MIN = 64, FX_E_MAX = 1960;  // exponent fields of a line that
 // Schedule R = 1 (two stages, one exchange; N = 2^p with p >= 7, else as R = 0):
 //   E = 2^ceil(p/2); a radix-E stage, then radix N/E (16.8 for 128, 16.16 for
 //   256, 32.16 for 512, 32.32 for 1024).  Four times the registers of R = 0
-//   for half the shared-memory exchanges: used by the complex64 y and z passes
-//   when the autotuner finds it faster.
-// Schedule R = 2 (N = 2^p with p >= 7, else as R = 0): E = 16; radix 16, 16, then
-//   N/256 (16.8 for 128): one exchange fewer than R = 0 and half its threads a
-//   line, for tiles twice as wide in the same CTA (complex64 pass A).
+//   for half the shared-memory exchanges: the complex64 y passes from n = 256 on
+//   by default, the others where the autotuner finds it faster.
+// Schedule R = 2 (N = 512 and 1024, else as R = 0): E = 16; radix 16, 16, then N/256:
+//   half the threads a line of R = 0, for tiles twice as wide in the same CTA
+//   (complex64 x passes).
+// Schedule R = 3 (the fixed-point lines): as R = 0, but with more than three stages
+//   the short one comes second (8, 2, 8, 8 for 1024), so that the last is of radix 8.
 template <int N, int R = 0> struct FftPlan {
   static constexpr bool R3 = N % 3 == 0;
   static constexpr int P2 = ilog2c(N);
   static constexpr bool TWO = R == 1 && !R3 && P2 >= 7;
-  static constexpr bool E16 = R == 2 && !R3 && P2 >= 7;
+  static constexpr bool E16 = R == 2 && !R3 && P2 >= 9;
   static constexpr int E = E16 ? 16 : TWO ? (1 << ((P2 + 1) / 2)) : (R3 ? 12 : 8);
   static constexpr int T = N / E;  // threads per line
   static constexpr int P = ilog2c(R3 ? N / 12 : N);
   static constexpr int Q = R3 ? P / 2 : P / 3;
   static constexpr int REM = R3 ? P % 2 : P % 3;
   static constexpr bool SHORT2 = R == 3 && !R3 && REM != 0 && Q > 2;  // the short stage second
-  static constexpr int S = E16 ? (P2 > 8 ? 3 : 2) : TWO ? 2 : (R3 ? 1 + Q + REM : Q + (REM ? 1 : 0));
+  static constexpr int S = E16 ? 3 : TWO ? 2 : (R3 ? 1 + Q + REM : Q + (REM ? 1 : 0));
   __host__ __device__ static constexpr int radix(int i) {
-    return E16 ? (i == 0 ? 16 : i == 1 ? (N < 256 ? N / 16 : 16) : N / 256)
+    return E16 ? (i < 2 ? 16 : N / 256)
            : TWO ? (i == 0 ? E : N / E) : R3 ? (i == 0 ? 12 : (i <= Q ? 4 : 2)) : (i == (SHORT2 ? 1 : Q) ? (REM == 1 ? 2 : 4) : 8);
   }
   __host__ __device__ static constexpr int ns(int i) { return i == 0 ? 1 : ns(i - 1) * radix(i - 1); }
 };
-
-// Schedule R = 3 (the fixed-point lines): as R = 0, but with more than three stages
-// the short one comes second (8, 2, 8, 8 for 1024), so that the last is of radix 8.
 
 // Complex constants in the representation of C.
 __device__ __forceinline__ double2 cconst(double re, double im, double2) { return double2{re, im}; }
@@ -993,8 +1000,8 @@ __device__ __forceinline__ void fft_line(typename A::C (&v)[FftPlan<N, R>::E], i
 }
 
 // Shared-memory views. Tile of CW columns of a strided axis: [pos][col] with a
-// row pitch of PITCH >= CW elements (off: where the column sits in a row).  (Rows of 64 bytes take twice the
-// minimum shared-memory wavefronts in the first exchange, where each thread
+// row pitch of PITCH >= CW elements (off: where the column sits in a row).  (Rows of 64
+// bytes take twice the minimum shared-memory wavefronts in the first exchange, where each thread
 // writes its E outputs E rows apart; a padding row every E rows removes that
 // but was measured slower at 512^3, by the index arithmetic it adds to every
 // access, so the tiles are unpadded.)  The columns of a tile interleave across
@@ -1006,7 +1013,7 @@ template <typename C, int CW, int T, int PITCH = CW> struct AccTile {
   static constexpr int G = CW >= 32 ? 1 : (32 / CW < T ? 32 / CW : T);  // threads of a column in a warp
   static constexpr int ROWS = T / G;                                       // partial maxima of a column
   static constexpr int MAXN = 2 * ROWS * CW;
-  static constexpr unsigned LANES = CW * T >= 32 ? 0xffffffffu : (1u << (CW * T % 32)) - 1;  // (tiles of under 32 threads)
+  static constexpr unsigned LANES = CW * T >= 32 ? 0xffffffffu : (1u << (CW * T % 32)) - 1;  // (small tiles)
   C* sm;
   int off, col;
   int* mxs;
@@ -1146,11 +1153,23 @@ template <typename C, int T> struct AccLineX {
 __host__ __device__ constexpr int ctas(int threads, int resident) {
   return resident / threads < 1 ? 1 : (resident / threads > 8 ? 8 : resident / threads);
 }
+// z pass, us without a bound, with 512, 768 and 1024: complex128 128^3 48.2 / 48.5 / 43.4 /
+// 41.3, 256^3 381 / 380 / 314 / 298, 512^3 4774 / 3397 / 2714 / 2479; double-float 96^3
+// 31.3 / 22.8 / 23.7 / 26.2, 192^3 209 / 171 / 168 / 179, 512^3 3498 / 2653 / 2540 / 2582
+// (64^3 and below alike; two groups are slower than one however bounded); complex64
+// 512^3 588 / 593 / 566 / 552, 1024^3 5583 / 5562 / 5582 / 5738, two groups 256^3 62.1 /
+// 61.9 / 57.4 / 65.7 (55.5 with 640), 512^3 475 / 475 / 492 / 592, 192^3 42.6 / 38.7 / 44.2 /
+// 46.2, two-stage 512^3 488 / 486 / 691 / 887 (488 with 384).
 template <class A, int N, int ZG, int R> constexpr int z_resident() {
   if (A::id == 0) return ZG == 1 ? 1024 : 1;
   if (A::id == 2) return ZG > 1 ? 1 : N == 96 ? 512 : N <= 64 ? 1024 : 768;
   return R == 1 ? 384 : N % 3 == 0 || (ZG > 1 && N >= 512) ? 512 : ZG == 1 ? 768 : 640;
 }
+// Projection, likewise: complex64 192^3 46.0 / 45.8 / 42.0 / 39.9, 256^3 120 / 120 / 120 / 93
+// (with lower states 314 / 314 / 314 / 195); complex128 256^3 463 / 463 / 411 / 404, 512^3
+// 4661 / 4662 / 4662 / 3498, with lower states 256^3 2138 / 1874 / 1855 / 1858; double-float
+// 96^3 20.2 / 17.5 / 20.4 / 24.5, 128^3 39.2 / 34.2 / 28.9 / 30.7, 256^3 313 / 234 / 202 / 211,
+// with lower states 96^3 69.9 / 40.7 / 45.7 / 53.5, 192^3 622 / 463 / 455 / 380.
 template <class A, int N, bool LOWER> constexpr int project_resident() {
   return A::id == 1 || (A::id == 0 && !LOWER) ? 1024 : A::id == 2 && !LOWER && N % 3 != 0 && N <= 256 ? 768 : 512;
 }
@@ -1568,8 +1587,9 @@ k_zpass(const __grid_constant__ BatchZ b) {
 // Measured us a step, separate passes then this one: complex64 16^3 6.95 and 3.92,
 // 64^3 9.85 and 7.41, 96^3 22.3 and 20.8, 128^3 33.1 and 29.8; complex128 32^3
 // 24.4 and 19.6, 64^3 31.0 and 39.9; double-float 32^3 15.4 and 13.5, 64^3 19.7
-// and 23.2 (the last of each pair is why the line is drawn at 32).  Each thread owns one radix column (E elements) of the plane, or GRP of them
-// in turn where the plane has more than 1024.
+// and 23.2 (the last of each pair is why the line is drawn at 32).  Each thread owns one
+// radix column (E elements) of the plane, or GRP of them in turn where the plane has more
+// than 1024.
 template <class A, int N> struct PlaneShape {
   static constexpr int T = N / FftPlan<N>::E;
   static constexpr size_t SMEM = (size_t)N * Shape<A, N>::LPAD * sizeof(typename A::C);
@@ -1725,7 +1745,7 @@ __device__ __forceinline__ void update_x_body(typename A::C* W, typename A::C* _
   if constexpr (STATS == STATS_FULL) full_store<A>(facc, part);
 }
 // Lattice i of the batch applies its pending normalisation factor when bit i
-// of `scaled` is set. 
+// of `scaled` is set.
 template <class A, int N, int STATS, int XC, int R = 0>
 __global__ void __launch_bounds__(FftPlan<N, R>::T * XC,
                                   ctas(FftPlan<N, R>::T * XC, x_resident<A, N, R>()))
